@@ -154,7 +154,7 @@ typedef struct {
                                  which saturates the host link even beside the
                                  replica's compute and leaves most of each SM
                                  to it; device-side launches give every
-                                 32 KiB unit its own warp or CTA.  With a cap,
+                                 piece of the work its own warp or CTA.  With a cap,
                                  each warp or CTA strides over many units       */
   uint32_t flags;             /* KVX_FLAG_*                                     */
   int64_t wait_cycles;        /* limit of every bounded wait inside a kernel, in

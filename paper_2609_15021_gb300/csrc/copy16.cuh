@@ -19,45 +19,18 @@ __device__ __forceinline__ void st16(uint8_t* p, const uint4& v) {
   __stcs(reinterpret_cast<uint4*>(p), v);
 }
 
-// Move kInflight vectors: pack reads the page side, unpack reads the chunk side.
-template <int DIR>
-__device__ __forceinline__ void move_batch(uint8_t* pg, uint8_t* ck, const int64_t (&po)[kInflight],
-                                           const int64_t (&co)[kInflight]) {
-  uint4 v[kInflight];
-  if (DIR == kPack) {
-#pragma unroll
-    for (int i = 0; i < kInflight; ++i) v[i] = ld16(pg + po[i]);
-#pragma unroll
-    for (int i = 0; i < kInflight; ++i) st16(ck + co[i], v[i]);
-  } else {
-#pragma unroll
-    for (int i = 0; i < kInflight; ++i) v[i] = ld16(ck + co[i]);
-#pragma unroll
-    for (int i = 0; i < kInflight; ++i) st16(pg + po[i], v[i]);
-  }
-}
-
-template <int DIR>
-__device__ __forceinline__ void move_one(uint8_t* pg, uint8_t* ck, int64_t po, int64_t co) {
-  if (DIR == kPack)
-    st16(ck + co, ld16(pg + po));
-  else
-    st16(pg + po, ld16(ck + co));
-}
-
-// Same byte order on both sides (NHD pages, opaque segments): a flat copy of
-// nbytes (a multiple of 16).
-template <int DIR>
-__device__ __forceinline__ void move_flat(uint8_t* pg, uint8_t* ck, int64_t nbytes, int lane) {
+// One warp's copy of nbytes (a multiple of 16).
+__device__ __forceinline__ void copy_flat(uint8_t* dst, const uint8_t* src, int64_t nbytes, int lane) {
   int64_t off = (int64_t)lane * 16;
   constexpr int64_t kStep = 32 * 16;
   for (; off + (kInflight - 1) * kStep < nbytes; off += kInflight * kStep) {
-    int64_t o[kInflight];
+    uint4 v[kInflight];
 #pragma unroll
-    for (int i = 0; i < kInflight; ++i) o[i] = off + i * kStep;
-    move_batch<DIR>(pg, ck, o, o);
+    for (int i = 0; i < kInflight; ++i) v[i] = ld16(src + off + i * kStep);
+#pragma unroll
+    for (int i = 0; i < kInflight; ++i) st16(dst + off + i * kStep, v[i]);
   }
-  for (; off < nbytes; off += kStep) move_one<DIR>(pg, ck, off, off);
+  for (; off < nbytes; off += kStep) st16(dst + off, ld16(src + off));
 }
 
 }  // namespace

@@ -17,13 +17,39 @@ constexpr int kMaxSegments = 96;  // segments per opaque-copy launch (params < 4
 
 enum Dir : int { kPack = 0, kUnpack = 1 };
 
-// One contiguous chunk-side region: layers [l0, l0 + nl) of one chunk.
+// Division of 32-bit unsigned numbers by a launch constant d >= 1: with
+// m = floor(2^64 / d) + 1, floor(n / d) is the high word of m * n for every
+// 32-bit n and d > 1 (Lemire, Kaser, Kurz, "Faster remainder by direct
+// computation", 2019).
+struct FastDiv {
+  uint64_t m;
+  uint32_t d;
+};
+inline FastDiv fast_div(uint32_t d) { return {d > 1 ? UINT64_MAX / d + 1 : 0, d}; }
+
+// One contiguous chunk-side region: layers [l0, l0 + nl) of one chunk.  Each
+// (layer, K|V) of it is a plane of `tokens` token rows, cut into
+// units_per_plane work units.
 struct Job {
   uint8_t* chunk;       // chunk-side address of layer l0 (device, staging or mapped host)
-  int64_t first_block;  // logical block index of the chunk's first token
+  int64_t first_entry;  // table entry (logical block) of the chunk's first token
   int64_t unit_end;     // exclusive prefix sum of units up to and including this job
+  int32_t first_sub;    // page of that entry's logical block that holds the token
   int32_t tokens;       // T_c: tokens held by the chunk
-  int32_t l0;           // first layer of the region
+  int32_t units_per_plane;
+  int16_t l0, nl;       // layers of the region
+};
+
+// Counters from which the warps of one launch of the load/store kernel take
+// their units one after another (`taken` null: each warp strides over the units
+// of its own).  They only count up, by what the launch is bound to add: *taken,
+// from `base`, by one for every unit, and taken[1], from done_base, by one for
+// every CTA that is done.  The last one writes `ticket` to *done in mapped host
+// memory, which tells the host that the counters may serve another launch.
+struct UnitQueue {
+  uint32_t* taken;
+  uint32_t* done;
+  uint32_t base, done_base, ticket;
 };
 
 // Kernel parameters of one pack/unpack launch (passed by value, < 4 KiB).
@@ -32,17 +58,21 @@ struct MoveParams {
   Job jobs[kMaxJobs];
   const int32_t* table;        // device block table
   long long* err;              // device error word (lowest bad logical block)
-  int64_t num_blocks;          // pages per layer
   int64_t page_bytes;          // 2 * H * B * row
   int64_t total_units;         // units of this launch
+  UnitQueue units;             // load/store kernel only
+  FastDiv by_row, by_heads, by_block, by_group;  // 16-byte vectors per row, H, B, ppb
+  uint32_t entries;            // valid table entries, as unsigned numbers, are below this
   int32_t n_jobs;
-  int32_t blocks_per_chunk;    // C / B: kernel pages per chunk
-  int32_t ppb;                 // pages per logical block named by the table (>= 1)
-  int32_t B, H, R;             // tokens per page, heads, row bytes
-  int32_t fast;                // 1 if R/16 is a power of two <= 32
-  int32_t vpr_shift;           // log2(R / 16) when fast
-  int32_t rpi_div_h, rpi_mod_h; // (32 / (R/16)) / H and % H when fast
+  uint32_t ppb;                // pages per logical block named by the table (>= 1)
+  uint32_t B, H, R;            // tokens per page, heads, row bytes
+  uint32_t head_step, tok_step; // rows of a page half from a head / token to the next
+  // 32 16-byte vectors, a warp's step: columns, heads, tokens of a page, pages of a
+  // logical block, logical blocks
+  uint32_t step_col, step_head, step_tok, step_sub, step_entry;
+  uint32_t unit_vectors;       // 16-byte vectors of a unit of the load/store kernel
 };
+static_assert(sizeof(MoveParams) <= 4096, "kernel parameters");
 
 // One contiguous byte range of an opaque copy (a recurrent-state slot).
 struct Segment {
@@ -80,14 +110,16 @@ enum Where : int { kHostChunks = 0, kDeviceChunks = 1 };
 kvx_status check_transfer(int device, const kvx_pool* P, const int32_t* table, int64_t table_len, int64_t t0,
                           int64_t t1, int32_t C, void* const* chunks, int64_t n_chunks, cudaStream_t stream,
                           int where, int mode, Geometry* g, int64_t* n, uint8_t** side);
-void init_params(MoveParams* p, long long* err, const kvx_pool* P, const Geometry& g, const int32_t* table,
-                 int32_t C);
-void push_job(MoveParams* p, uint8_t* chunk_side, int64_t first_block, int32_t tokens, int32_t l0, int32_t nl);
+void init_params(MoveParams* p, long long* err, const kvx_pool* P, const Geometry& g, const int32_t* table);
+void push_job(MoveParams* p, uint8_t* chunk_side, int64_t first_page, int32_t tokens, int32_t l0, int32_t nl);
+// Cuts the jobs of `p` into units for launch_move; returns the CTAs that give
+// every unit a warp of its own.  link: the chunks are mapped host memory.
+int64_t cut_units(MoveParams* p, bool link);
 int64_t chunk_bytes(const kvx_pool* P, const Geometry& g, int64_t tokens);
 void set_error_text(const char* text);
 
 // Launchers (pack_kernels.cu).  Return the cudaError_t of the launch.
-cudaError_t launch_move(int dir, int layout, const MoveParams& p, int grid, cudaStream_t s);
+cudaError_t launch_move(int dir, const MoveParams& p, int grid, cudaStream_t s);
 cudaError_t launch_segments(const SegmentParams& p, int grid, cudaStream_t s);
 // Loads the pack kernels into the current context if lazy loading has not yet.
 cudaError_t load_pack_kernels();
@@ -114,7 +146,7 @@ constexpr int kTensorMapBytes = 128;
 bool encode_tensor_maps(const kvx_pool* P, int64_t row_bytes, void* out);
 cudaError_t launch_move_tmap(int dir, const MoveParams& p, const void* maps, int num_layers, int grid,
                              int stage_bytes, int stages, const TmaWait& wt, cudaStream_t s);
-int move_ctas_per_sm(int dir, int layout);
+int move_ctas_per_sm(int dir);
 int segment_ctas_per_sm();
 // Shared tier (tier_kernels.cu): publication of up to kMaxPublish commits in
 // one launch.  Thread j makes a system-scope release store of seq0 + j to the

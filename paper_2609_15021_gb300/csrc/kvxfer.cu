@@ -99,6 +99,11 @@ constexpr int32_t kDefaultSlots = 4;
 // carrying its layers' tensor maps).
 constexpr int64_t kDefaultSlotBytes = 128ll << 20;
 constexpr long long kNoError = LLONG_MAX;
+// Launches over the host link take their units from a queue (UnitQueue) from
+// this many units a warp on; below it warps hardly drift apart.
+constexpr int64_t kQueueRounds = 8;
+// More than the launches the driver lets a host thread run ahead by (1024).
+constexpr uint32_t kUnitQueues = 1280;
 
 struct TimedLaunch {
   cudaEvent_t a, b;
@@ -114,7 +119,7 @@ struct kvx_ctx {
   int32_t store_mode = KVX_MODE_STAGED;
   int32_t load_mode = KVX_MODE_STAGED;
   int num_sms = 1;
-  int move_occ[2][2] = {{1, 1}, {1, 1}};
+  int move_occ[2] = {1, 1};
   int seg_occ = 1;
   int link_ctas = 1;  // default CTA cap of launches that cross the host link
   cudaStream_t s_kern = nullptr;  // pack / unpack kernels
@@ -131,6 +136,11 @@ struct kvx_ctx {
   int32_t next_slot = 0;
   long long* d_err = nullptr;  // 16-byte allocation: error word, then the timeout flag
   int* d_timeout = nullptr;
+  uint32_t* d_queues = nullptr;    // kUnitQueues x (units taken, CTAs done)
+  uint32_t* queue_done = nullptr;  // pinned: ticket of the last launch that is done with queue i
+  uint32_t* queue_done_dev = nullptr;
+  std::vector<UnitQueue> queues;  // as the next launch gets them; ticket: of the last one
+  uint32_t next_queue = 0;
   std::mutex mu;
   // end of this context's last transfer call (host clock, ns), for the host touch
   int64_t last_call_ns = 0;
@@ -320,10 +330,38 @@ const void* tensor_maps_of(kvx_ctx* ctx, const kvx_pool* P, int64_t row) {
   return ctx->tmap_ok ? tensor_map_storage(ctx) : nullptr;
 }
 
+// Cuts the jobs into one unit per page half for the TMA kernels, one CTA each.
+int64_t cut_pages(MoveParams* p) {
+  p->total_units = 0;
+  for (int32_t i = 0; i < p->n_jobs; ++i) {
+    Job& J = p->jobs[i];
+    J.units_per_plane = (J.tokens + p->B - 1) / p->B;
+    p->total_units += 2ll * J.nl * J.units_per_plane;
+    J.unit_end = p->total_units;
+  }
+  return p->total_units;
+}
+
+// Unit queue for a launch on `s`, or none: when the stream is being captured (a
+// replay would use the queue at times the host does not see), or when the
+// launch that had the queue last is not done.
+UnitQueue* take_unit_queue(kvx_ctx* ctx, cudaStream_t s) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  if (cap != cudaStreamCaptureStatusNone) return nullptr;
+  const uint32_t i = ctx->next_queue;
+  ctx->next_queue = (i + 1) % kUnitQueues;
+  UnitQueue* q = &ctx->queues[i];
+  return __atomic_load_n(ctx->queue_done + i, __ATOMIC_ACQUIRE) == q->ticket ? q : nullptr;
+}
+
 // Launch one pack/unpack kernel with optional timing events around it.
 // over_link: the launch reads or writes mapped host memory, so the host link,
 // not HBM, bounds it and a fraction of the SMs saturates it.
-kvx_status launch_move_timed(kvx_ctx* ctx, const kvx_pool* P, int dir, int layout, const MoveParams& p,
+kvx_status launch_move_timed(kvx_ctx* ctx, const kvx_pool* P, int dir, int layout, MoveParams& p,
                              int64_t bytes, cudaStream_t s, bool over_link) {
   // TMA variants: device-side chunks only, and a K or V half page (the
   // largest unit) of at most 48 KiB: one shared-memory stage per unit, or a
@@ -343,13 +381,16 @@ kvx_status launch_move_timed(kvx_ctx* ctx, const kvx_pool* P, int dir, int layou
   // DRAM busier than a persistent grid walking the units in lockstep.
   // Launches over the host link, or capped by the caller (max_ctas), are
   // persistent: each warp or CTA strides over many units.
-  int64_t grid = tma ? p.total_units : (p.total_units + (kThreads / 32) - 1) / (kThreads / 32);
-  int64_t cap = grid;
+  int64_t cap = INT_MAX;  // grid.x limit
   if (ctx->opts.max_ctas > 0)
     cap = ctx->opts.max_ctas;
   else if (over_link)
-    cap = std::min<int64_t>(ctx->link_ctas, (int64_t)ctx->num_sms * ctx->move_occ[dir][layout]);
-  grid = std::max<int64_t>(1, std::min(std::min(grid, cap), (int64_t)INT_MAX));  // grid.x limit
+    cap = std::min<int64_t>(ctx->link_ctas, (int64_t)ctx->num_sms * ctx->move_occ[dir]);
+  const int64_t wanted = tma ? cut_pages(&p) : cut_units(&p, over_link);
+  const int64_t grid = std::max<int64_t>(1, std::min(wanted, cap));
+  UnitQueue* queue = over_link && wanted >= kQueueRounds * grid ? take_unit_queue(ctx, s) : nullptr;
+  p.units = queue ? *queue : UnitQueue{};
+  p.units.ticket++;
   int stage_bytes = 0, stages = 0;
   if (tma) {
     // one stage when each CTA moves one unit; else a ring of 3 (2 above 32 KiB)
@@ -373,7 +414,12 @@ kvx_status launch_move_timed(kvx_ctx* ctx, const kvx_pool* P, int dir, int layou
   else if (tma)
     KVX_CUDA_AT("launch", launch_move_tma(dir, layout, p, (int)grid, stage_bytes, stages, wt, s));
   else
-    KVX_CUDA_AT("launch", launch_move(dir, layout, p, (int)grid, s));
+    KVX_CUDA_AT("launch", launch_move(dir, p, (int)grid, s));
+  if (queue) {
+    queue->base += (uint32_t)p.total_units;
+    queue->done_base += (uint32_t)grid;
+    queue->ticket++;
+  }
   ctx->launches++;
   if (timing && a && b) {
     KVX_CUDA(cudaEventRecord(b, s));
@@ -382,29 +428,34 @@ kvx_status launch_move_timed(kvx_ctx* ctx, const kvx_pool* P, int dir, int layou
   return KVX_OK;
 }
 
-void init_move_params(MoveParams* p, long long* err, const kvx_pool* P, const Geometry& g,
-                      const int32_t* table, int32_t C) {
+void init_move_params(MoveParams* p, long long* err, const kvx_pool* P, const Geometry& g, const int32_t* table) {
   memset(p, 0, sizeof(*p));
   for (int l = 0; l < P->num_layers; ++l) p->layer_base[l] = (uint8_t*)P->layer_base[l];
   p->table = table;
   p->err = err;
-  p->num_blocks = P->num_blocks;
-  p->page_bytes = g.page_bytes;
-  p->blocks_per_chunk = C / P->block_tokens;
   p->ppb = pages_per_block(P);
+  p->entries = (uint32_t)std::min<int64_t>(P->num_blocks / p->ppb, 1ll << 31);  // an int32 names no more
+  p->page_bytes = g.page_bytes;
   p->B = P->block_tokens;
   p->H = P->num_heads;
   p->R = (int32_t)g.row;
-  const int64_t vpr = g.row / 16;
-  p->fast = (vpr >= 1 && vpr <= 32 && (vpr & (vpr - 1)) == 0) ? 1 : 0;
-  if (p->fast) {
-    int sh = 0;
-    while ((1ll << sh) < vpr) ++sh;
-    p->vpr_shift = sh;
-    const int rows_per_step = 32 >> sh;
-    p->rpi_div_h = rows_per_step / P->num_heads;
-    p->rpi_mod_h = rows_per_step % P->num_heads;
-  }
+  p->head_step = P->layout == KVX_LAYOUT_HND ? p->B : 1;
+  p->tok_step = P->layout == KVX_LAYOUT_HND ? 1 : p->H;
+  uint32_t step = 32;
+  const auto split = [&step](uint32_t n) {
+    const uint32_t rest = step % n;
+    step /= n;
+    return rest;
+  };
+  p->step_col = split((uint32_t)(g.row / 16));
+  p->step_head = split(p->H);
+  p->step_tok = split(p->B);
+  p->step_sub = split(p->ppb);
+  p->step_entry = step;
+  p->by_row = fast_div((uint32_t)(g.row / 16));
+  p->by_heads = fast_div((uint32_t)p->H);
+  p->by_block = fast_div((uint32_t)p->B);
+  p->by_group = fast_div((uint32_t)p->ppb);
 }
 
 // A chunk-side region of one launch: layers [l0, l0+nl) of chunk i.
@@ -414,17 +465,15 @@ struct Piece {
   int64_t bytes;   // nl * 2 * T_i * H * row
 };
 
-void add_job(MoveParams* p, uint8_t* chunk_side, int64_t first_block, int32_t tokens, int32_t l0,
-             int32_t nl) {
-  Job& J = p->jobs[p->n_jobs];
+// first_page: page (in token order) of the chunk's first token.
+void add_job(MoveParams* p, uint8_t* chunk_side, int64_t first_page, int32_t tokens, int32_t l0, int32_t nl) {
+  Job& J = p->jobs[p->n_jobs++];
   J.chunk = chunk_side;
-  J.first_block = first_block;
+  J.first_entry = first_page / p->ppb;
+  J.first_sub = (int32_t)(first_page % p->ppb);
   J.tokens = tokens;
-  J.l0 = l0;
-  const int64_t units = (int64_t)nl * p->blocks_per_chunk * 2;
-  p->total_units += units;
-  J.unit_end = p->total_units;
-  p->n_jobs++;
+  J.l0 = (int16_t)l0;
+  J.nl = (int16_t)nl;
 }
 
 kvx_status ensure_staging(kvx_ctx* ctx) {
@@ -462,7 +511,7 @@ struct Plan {
 // stream s.
 kvx_status enqueue_direct(kvx_ctx* ctx, const Plan& pl, cudaStream_t s) {
   MoveParams p;
-  init_move_params(&p, ctx->d_err, pl.P, pl.g, pl.table, pl.C);
+  init_move_params(&p, ctx->d_err, pl.P, pl.g, pl.table);
   int64_t bytes = 0;
   for (int64_t i = 0; i < pl.n; ++i) {
     add_job(&p, pl.side[i], (pl.first_chunk + i) * pl.bpc, pl.tokens[i], 0, pl.P->num_layers);
@@ -472,7 +521,6 @@ kvx_status enqueue_direct(kvx_ctx* ctx, const Plan& pl, cudaStream_t s) {
       kvx_status st = launch_move_timed(ctx, pl.P, pl.dir, pl.P->layout, p, bytes, s, pl.over_link);
       if (st != KVX_OK) return st;
       p.n_jobs = 0;
-      p.total_units = 0;
       bytes = 0;
     }
   }
@@ -496,7 +544,7 @@ kvx_status enqueue_staged(kvx_ctx* ctx, const Plan& pl) {
     ctx->next_slot = (ctx->next_slot + 1) % ctx->nslots;
     uint8_t* slot = ctx->slots[k];
     MoveParams p;
-    init_move_params(&p, ctx->d_err, P, pl.g, pl.table, pl.C);
+    init_move_params(&p, ctx->d_err, P, pl.g, pl.table);
     int64_t off = 0;
     for (const Piece& pc : batch) {
       add_job(&p, slot + off, (pl.first_chunk + pc.i) * pl.bpc, pl.tokens[pc.i], pc.l0, pc.nl);
@@ -634,13 +682,12 @@ kvx_status check_transfer(int device, const kvx_pool* P, const int32_t* table, i
   return KVX_OK;
 }
 
-void init_params(MoveParams* p, long long* err, const kvx_pool* P, const Geometry& g, const int32_t* table,
-                 int32_t C) {
-  init_move_params(p, err, P, g, table, C);
+void init_params(MoveParams* p, long long* err, const kvx_pool* P, const Geometry& g, const int32_t* table) {
+  init_move_params(p, err, P, g, table);
 }
 
-void push_job(MoveParams* p, uint8_t* chunk_side, int64_t first_block, int32_t tokens, int32_t l0, int32_t nl) {
-  add_job(p, chunk_side, first_block, tokens, l0, nl);
+void push_job(MoveParams* p, uint8_t* chunk_side, int64_t first_page, int32_t tokens, int32_t l0, int32_t nl) {
+  add_job(p, chunk_side, first_page, tokens, l0, nl);
 }
 
 int64_t chunk_bytes(const kvx_pool* P, const Geometry& g, int64_t tokens) { return chunk_bytes_of(P, g, tokens); }
@@ -837,6 +884,8 @@ void destroy_ctx(kvx_ctx* ctx) {
     if (ctx->ev_kern_done) cudaEventDestroy(ctx->ev_kern_done);
     if (ctx->ev_copy_done) cudaEventDestroy(ctx->ev_copy_done);
     if (ctx->d_err) cudaFree(ctx->d_err);
+    if (ctx->d_queues) cudaFree(ctx->d_queues);
+    if (ctx->queue_done) cudaFreeHost(ctx->queue_done);
     if (ctx->s_kern) cudaStreamDestroy(ctx->s_kern);
     if (ctx->s_copy) cudaStreamDestroy(ctx->s_copy);
     if (ctx->s_aux) cudaStreamDestroy(ctx->s_aux);
@@ -942,8 +991,18 @@ kvx_status kv_ctx_create(int device, const kvx_opts* opts, kvx_ctx** out) {
     ctx->d_timeout = reinterpret_cast<int*>(ctx->d_err + 1);
     const long long init[2] = {kNoError, 0};
     if ((e = cudaMemcpy(ctx->d_err, init, sizeof(init), cudaMemcpyHostToDevice)) != cudaSuccess) return fail(e);
-    for (int d = 0; d < 2; ++d)
-      for (int l = 0; l < 2; ++l) ctx->move_occ[d][l] = move_ctas_per_sm(d, l);
+    if ((e = cudaMalloc(&ctx->d_queues, kUnitQueues * 2 * sizeof(uint32_t))) != cudaSuccess) return fail(e);
+    if ((e = cudaMemsetAsync(ctx->d_queues, 0, kUnitQueues * 2 * sizeof(uint32_t), ctx->s_aux)) != cudaSuccess ||
+        (e = cudaStreamSynchronize(ctx->s_aux)) != cudaSuccess)
+      return fail(e);
+    if ((e = cudaHostAlloc(&ctx->queue_done, kUnitQueues * sizeof(uint32_t), cudaHostAllocMapped)) != cudaSuccess ||
+        (e = cudaHostGetDevicePointer((void**)&ctx->queue_done_dev, ctx->queue_done, 0)) != cudaSuccess)
+      return fail(e);
+    memset(ctx->queue_done, 0, kUnitQueues * sizeof(uint32_t));
+    ctx->queues.resize(kUnitQueues);
+    for (uint32_t i = 0; i < kUnitQueues; ++i)
+      ctx->queues[i] = {ctx->d_queues + 2 * i, ctx->queue_done_dev + i, 0, 0, 0};
+    for (int d = 0; d < 2; ++d) ctx->move_occ[d] = move_ctas_per_sm(d);
     ctx->seg_occ = segment_ctas_per_sm();
     if ((e = prepare_tma_kernels()) != cudaSuccess) return fail(e);
     // the host-page touch threads, once per process, at set-up rather than

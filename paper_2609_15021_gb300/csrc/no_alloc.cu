@@ -181,7 +181,7 @@ extern "C" kvx_status kv_store_noalloc(const kvx_pool* pool, const int32_t* bloc
     auto flush = [&]() -> kvx_status {
       if (nb == 0) return KVX_OK;
       MoveParams p;
-      init_params(&p, err, pool, g, block_table, chunk_tokens);
+      init_params(&p, err, pool, g, block_table);
       int64_t off = 0;
       for (int q = 0; q < nb; ++q) {
         push_job(&p, staging + off, (first_chunk + batch[q].i) * bpc, (int32_t)tokens_of(batch[q].i), batch[q].l0,
@@ -189,8 +189,8 @@ extern "C" kvx_status kv_store_noalloc(const kvx_pool* pool, const int32_t* bloc
         off += batch[q].bytes;
       }
       // one warp per unit, as for the library's other HBM-bound launches
-      const int64_t grid = std::max<int64_t>(1, (p.total_units + kThreads / 32 - 1) / (kThreads / 32));
-      cudaError_t le = launch_move(kPack, pool->layout, p, (int)grid, stream);
+      const int64_t grid = std::max<int64_t>(1, cut_units(&p, false));
+      cudaError_t le = launch_move(kPack, p, (int)grid, stream);
       if (le != cudaSuccess) return fail_cuda(le, "pack kernel launch");
       int64_t soff = 0;
       for (int q = 0; q < nb;) {

@@ -7,17 +7,20 @@
 // and staging, the host link for mapped pinned chunks), so it runs on the
 // load/store units with 16-byte vectors; no tensor cores are involved.
 //
-// Work unit: one (chunk, layer, page, K|V) region, handled by one warp.  For
-// the shapes of a 27B-class model (B = 16 tokens, H = 8 heads, 256-byte rows)
-// a unit is 32 KiB: both its page side and its chunk side are contiguous
-// 32 KiB extents, the chunk side in [token][head] row order and the page side
-// in [head][token] order (HND) or [token][head] order (NHD).  Every 256-byte
-// row is read and written whole by 16 lanes, so each 128-byte line is used in
-// full on both sides.  Each lane keeps kInflight 16-byte loads in flight
-// before storing them.
+// Work unit: one batch, 4 KiB of one plane -- one (chunk, layer, K|V) -- handled
+// by one warp, kInflight 16-byte vectors per lane; where HBM bounds a large
+// launch, two batches.  The chunk side of a
+// plane is one contiguous extent in [token][head][row] order, so a unit is
+// contiguous there whatever the page and row sizes are, and its vectors are
+// found on the page side ([head][token] order for HND, [token][head] for NHD)
+// one by one: vector -> row -> (token, head) -> page of the block table ->
+// address.  A lane finds its first vector by divisions by launch constants
+// (FastDiv) and the others by steps of 32 vectors, with carries.  A unit may
+// start and end inside a row or a page and may span pages.
 //
-// Out-of-range block-table entries skip their unit and lower a device error
-// word (atomicMin of the logical block index); nothing traps.
+// Out-of-range block-table entries skip their vectors (a pack writes zeros)
+// and lower a device error word (atomicMin of the logical block index);
+// nothing traps.
 
 #include "copy16.cuh"
 #include "kvx_internal.h"
@@ -25,150 +28,161 @@
 namespace kvx {
 namespace {
 
-// HND page side [H][B][R] <-> chunk side [nb][H][R], nr = nb * H rows, when
-// R / 16 is a power of two no larger than 32: a warp covers 32 / (R/16) whole
-// rows per step, each lane a fixed 16-byte column, and the (token, head) pair
-// of a lane's row is advanced incrementally (no division in the loop).
-template <int DIR>
-__device__ __forceinline__ void move_hnd_fast(uint8_t* pg, uint8_t* ck, int nr, const MoveParams& p,
-                                              int lane) {
-  const int rows_per_step = 32 >> p.vpr_shift;
-  const int64_t col = (int64_t)(lane & ((1 << p.vpr_shift) - 1)) * 16;
-  const int64_t R = p.R, B = p.B;
-  const int H = p.H;
-  int r = lane >> p.vpr_shift;  // row in chunk order: r = s * H + h
-  int s = r / H;
-  int h = r - s * H;
-  while (r + (kInflight - 1) * rows_per_step < nr) {
-    int64_t po[kInflight], co[kInflight];
-#pragma unroll
-    for (int i = 0; i < kInflight; ++i) {
-      po[i] = ((int64_t)h * B + s) * R + col;
-      co[i] = (int64_t)r * R + col;
-      r += rows_per_step;
-      s += p.rpi_div_h;
-      h += p.rpi_mod_h;
-      if (h >= H) {
-        h -= H;
-        ++s;
-      }
-    }
-    move_batch<DIR>(pg, ck, po, co);
-  }
-  while (r < nr) {
-    move_one<DIR>(pg, ck, ((int64_t)h * B + s) * R + col, (int64_t)r * R + col);
-    r += rows_per_step;
-    s += p.rpi_div_h;
-    h += p.rpi_mod_h;
-    if (h >= H) {
-      h -= H;
-      ++s;
-    }
-  }
+constexpr int kBatchVectors = 32 * kInflight;  // 4 KiB
+// Where HBM bounds a launch of more batches than this (32 MiB, about two for
+// each warp the GPU holds), a unit is two batches.  Packing 1 GB of 16-token
+// pages with one head of 256-byte rows took 337 us with units of one batch, 322
+// of two, 333 of four; with 8 heads 316, 300 and 306; packing 4 MB 9, 9 and 13 us.
+constexpr int64_t kBatchesApart = 8192;
+
+__device__ __forceinline__ uint32_t div_by(uint32_t n, const FastDiv& f) {
+  return f.d == 1 ? n : (uint32_t)__umul64hi(f.m, n);
+}
+__device__ __forceinline__ uint64_t div_by(uint64_t n, const FastDiv& f) {
+  return n >> 32 ? n / f.d : div_by((uint32_t)n, f);
 }
 
-// HND for any row size that is a multiple of 16 bytes.
+// What bounds it: the host link where the chunks are mapped host memory, HBM
+// where they are in device memory; either needs enough loads on their way.
+// Over the link a launch runs on some of the SMs, and these get unequal shares of
+// the link: which SMs they are, and so which CTAs fall behind, differs from one
+// GPU to another.  With units dealt out in advance a 1 GB restore took 4850 us
+// or up to 4955 (a store 5295 or up to 5370), depending on the GPU and the
+// number of CTAs; taking units from a queue it takes 4846 to 4849 (5294) on all
+// of them, with 48 CTAs as with 96.
+// Measured on GB300, one launch, 32 layers, 16-token HND pages, 8 heads of
+// head_dim 128 bf16 unless stated; in brackets the same call when a unit was a
+// page half, read row by row (vector by vector where a row was no power of two):
+//   restore over the link, 1 GB: 4848 us, 0.999 of the copy engines' 211.6 GB/s
+//     (4853 to 4890); head_dim 96, 256 MB: 1221 us (1335); one 128-byte head:
+//     1227 us (1263)
+//   restore, 4 MB: 27 us (32; head_dim 96: 107); 1 MB: 13 us (19; 60), since 4 KiB
+//     units put 256 warps on 1 MB where 32 of them made eight round trips each
+//   store over the link, 1 GB: 5294 us, 0.999 of 193.5 GB/s (5296); head_dim 96,
+//     256 MB: 1329 us (1508); one 128-byte head: 1334 us (1455)
+//   pack / unpack in device memory, 1 GB: 300 / 298 us, 6.8 TB/s (308 / 310);
+//     head_dim 96: 304 / 304 us (476 / 451); one 128-byte head: 350 / 354 (606 / 600)
+// Over the link a unit is one batch: units of eight (32 KiB a warp) took 4945 us
+// for the 1 GB restore and 5370 for the store, and equal shares of 26,368 B, so
+// that a warp's last batch is not whole, 95 us for a 16 MB restore instead of 83.
+// 80 registers, 3 CTAs per SM; at 64 it spills 48 bytes, and unpacking 1 GB into
+// HBM takes 310 us.
 template <int DIR>
-__device__ __forceinline__ void move_hnd_generic(uint8_t* pg, uint8_t* ck, int nr, const MoveParams& p,
-                                                 int lane) {
-  const int vpr = p.R / 16;
-  const int64_t nv = (int64_t)nr * vpr;
-  for (int64_t v = lane; v < nv; v += 32) {
-    const int64_t r = v / vpr;
-    const int64_t c = (v - r * vpr) * 16;
-    const int64_t s = r / p.H;
-    const int64_t h = r - s * p.H;
-    move_one<DIR>(pg, ck, (h * p.B + s) * p.R + c, r * p.R + c);
-  }
-}
-
-// At most 64 registers (4 CTAs of 256 threads per SM); no variant spills.
-template <int DIR, int LAYOUT>
-__global__ void __launch_bounds__(kThreads, 4) move_kernel(const __grid_constant__ MoveParams p) {
-  const int lane = threadIdx.x & 31;
-  const int64_t nwarps = ((int64_t)gridDim.x * kThreads) >> 5;
-  int64_t u = ((int64_t)blockIdx.x * kThreads + threadIdx.x) >> 5;
+__global__ void __launch_bounds__(kThreads, 3) move_kernel(const __grid_constant__ MoveParams p) {
+  const uint32_t lane = threadIdx.x & 31;
+  const uint32_t nwarps = gridDim.x * (kThreads / 32);
+  uint32_t job_begin = 0;
   int j = 0;
-  int64_t job_begin = 0;
-  const int64_t half_page = p.page_bytes >> 1;  // K or V part of a page: H * B * R
-  const int64_t HR = (int64_t)p.H * p.R;
-  for (; u < p.total_units; u += nwarps) {
+  uint32_t u = (blockIdx.x * kThreads + threadIdx.x) >> 5;
+  while (u < p.total_units) {
+    uint32_t next = u;  // taken now, so that the answer is there when this unit is done
+    if (p.units.taken && lane == 0) next = atomicAdd(p.units.taken, 1u) - p.units.base;
     while (u >= p.jobs[j].unit_end) {  // warp-uniform; units ascend per warp
       job_begin = p.jobs[j].unit_end;
       ++j;
     }
     const Job& J = p.jobs[j];
-    const int64_t local = u - job_begin;
-    const int kv = (int)(local & 1);
-    const int64_t rest = local >> 1;
-    const int jb = (int)(rest % p.blocks_per_chunk);
-    const int l = J.l0 + (int)(rest / p.blocks_per_chunk);
-    const int tok0 = jb * p.B;
-    if (tok0 >= J.tokens) continue;  // past the end of a short last chunk
-    const int nb = min(p.B, J.tokens - tok0);
-    // kernel page of the unit, the logical block naming it, and the pool page
-    const int64_t kpage = J.first_block + jb;
-    const int64_t lblk = kpage / p.ppb;
-    const int32_t entry = __ldg(p.table + lblk);
-    const int64_t page = (int64_t)entry * p.ppb + (kpage - lblk * p.ppb);
-    uint8_t* ck = J.chunk + ((int64_t)(l - J.l0) * 2 + kv) * J.tokens * HR + (int64_t)tok0 * HR;
-    const int nr = nb * p.H;
-    if (entry < 0 || (int64_t)entry >= p.num_blocks / p.ppb) {
-      if (lane == 0) atomicMin(p.err, (long long)lblk);
-      if (DIR == kPack) {  // the unit's chunk rows (contiguous) read as zeros
-        const uint4 z = make_uint4(0, 0, 0, 0);
-        for (int64_t off = (int64_t)lane * 16; off < (int64_t)nr * p.R; off += 32 * 16) st16(ck + off, z);
+    const uint32_t plane = (u - job_begin) / J.units_per_plane;  // (layer - l0) * 2 + kv
+    const uint64_t vectors = (uint64_t)J.tokens * p.H * p.by_row.d;  // of the plane
+    const uint64_t first = (uint64_t)(u - job_begin - plane * J.units_per_plane) * p.unit_vectors + lane;
+    // this lane's vectors: nv of them, 32 apart (none past the end of the plane)
+    int nv = first >= vectors ? 0 : (int)(min((uint64_t)p.unit_vectors, vectors - first + 31) >> 5);
+    uint8_t* ck = J.chunk + (plane * vectors + first) * 16;
+    uint8_t* base = p.layer_base[J.l0 + (plane >> 1)] + (plane & 1 ? p.page_bytes >> 1 : 0);
+    // place of the first vector: column of its row, head, token of its page, page
+    // of its logical block, table entry
+    const uint64_t row = div_by(first, p.by_row), tok = div_by(row, p.by_heads);
+    const uint32_t page = div_by((uint32_t)tok, p.by_block), gp = J.first_sub + page;
+    uint32_t col = (uint32_t)(first - row * p.by_row.d), h = (uint32_t)(row - tok * p.H);
+    uint32_t sp = (uint32_t)tok - page * p.B, e = div_by(gp, p.by_group), sub = gp - e * p.ppb;
+    const int32_t* entries = p.table + J.first_entry;
+    for (; nv > 0; nv -= kInflight, ck += kInflight * 512) {
+      uint4 data[kInflight];
+      if (DIR == kUnpack) {
+#pragma unroll
+        for (int i = 0; i < kInflight; ++i)
+          if (i < nv) data[i] = ld16(ck + i * 512);
       }
-      continue;
+#pragma unroll
+      for (int i = 0; i < kInflight; ++i) {
+        if (i < nv) {
+          const uint32_t entry = (uint32_t)__ldg(entries + e);
+          const bool ok = entry < p.entries;
+          const int64_t in_page = (int64_t)(h * p.head_step + sp * p.tok_step) * p.R + col * 16;
+          uint8_t* pg = base + ((int64_t)entry * p.ppb + sub) * p.page_bytes + in_page;
+          if (DIR == kPack) {
+            data[i] = make_uint4(0, 0, 0, 0);
+            if (ok) data[i] = ld16(pg);
+          } else if (ok) {
+            st16(pg, data[i]);
+          }
+          // reported once for each plane, by the page's first vector
+          if (!ok && in_page == 0) atomicMin(p.err, (long long)(J.first_entry + e));
+        }
+        // 32 vectors on
+        col += p.step_col;
+        h += p.step_head;
+        sp += p.step_tok;
+        sub += p.step_sub;
+        e += p.step_entry;
+        if (col >= p.by_row.d) col -= p.by_row.d, ++h;
+        if (h >= p.H) h -= p.H, ++sp;
+        if (sp >= p.B) sp -= p.B, ++sub;
+        if (sub >= p.ppb) sub -= p.ppb, ++e;
+      }
+      if (DIR == kPack) {
+#pragma unroll
+        for (int i = 0; i < kInflight; ++i)
+          if (i < nv) st16(ck + i * 512, data[i]);
+      }
     }
-    uint8_t* pg = p.layer_base[l] + (int64_t)page * p.page_bytes + kv * half_page;
-    if (LAYOUT == KVX_LAYOUT_NHD)
-      move_flat<DIR>(pg, ck, (int64_t)nr * p.R, lane);
-    else if (p.fast)
-      move_hnd_fast<DIR>(pg, ck, nr, p, lane);
-    else
-      move_hnd_generic<DIR>(pg, ck, nr, p, lane);
+    u = nwarps + (p.units.taken ? __shfl_sync(0xffffffffu, next, 0) : u);
   }
+  if (!p.units.taken) return;
+  __syncthreads();  // the warps of this CTA have taken their last units, and have the answers
+  if (threadIdx.x == 0 && atomicAdd(p.units.taken + 1, 1u) - p.units.done_base == gridDim.x - 1)
+    asm volatile("st.relaxed.sys.global.u32 [%0], %1;" ::"l"(p.units.done), "r"(p.units.ticket) : "memory");
 }
 
-template <int DIR, int LAYOUT>
-int occupancy_of() {
-  int n = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, move_kernel<DIR, LAYOUT>, kThreads, 0) !=
-      cudaSuccess) {
-    cudaGetLastError();
-    return 1;
-  }
-  return n > 0 ? n : 1;
-}
+using MoveKernel = void (*)(MoveParams);
+MoveKernel kernel_of(int dir) { return dir == kPack ? move_kernel<kPack> : move_kernel<kUnpack>; }
 
 }  // namespace
 
-cudaError_t launch_move(int dir, int layout, const MoveParams& p, int grid, cudaStream_t s) {
-  if (dir == kPack && layout == KVX_LAYOUT_HND)
-    move_kernel<kPack, KVX_LAYOUT_HND><<<grid, kThreads, 0, s>>>(p);
-  else if (dir == kPack)
-    move_kernel<kPack, KVX_LAYOUT_NHD><<<grid, kThreads, 0, s>>>(p);
-  else if (layout == KVX_LAYOUT_HND)
-    move_kernel<kUnpack, KVX_LAYOUT_HND><<<grid, kThreads, 0, s>>>(p);
-  else
-    move_kernel<kUnpack, KVX_LAYOUT_NHD><<<grid, kThreads, 0, s>>>(p);
+int64_t cut_units(MoveParams* p, bool link) {
+  const auto vectors = [p](const Job& J) { return (int64_t)J.tokens * p->H * p->by_row.d; };
+  int64_t batches = 0;  // of the launch
+  for (int32_t i = 0; i < p->n_jobs; ++i) batches += 2ll * p->jobs[i].nl * vectors(p->jobs[i]) / kBatchVectors;
+  p->unit_vectors = (link || batches <= kBatchesApart ? 1 : 2) * kBatchVectors;
+  p->total_units = 0;
+  for (int32_t i = 0; i < p->n_jobs; ++i) {
+    Job& J = p->jobs[i];
+    J.units_per_plane = (int32_t)((vectors(J) + p->unit_vectors - 1) / p->unit_vectors);
+    p->total_units += 2ll * J.nl * J.units_per_plane;
+    J.unit_end = p->total_units;
+  }
+  constexpr int64_t kWarps = kThreads / 32;
+  return (p->total_units + kWarps - 1) / kWarps;
+}
+
+cudaError_t launch_move(int dir, const MoveParams& p, int grid, cudaStream_t s) {
+  kernel_of(dir)<<<grid, kThreads, 0, s>>>(p);
   return cudaGetLastError();
 }
 
 cudaError_t load_pack_kernels() {
   // cudaFuncGetAttributes makes CUDA load a kernel that lazy loading has not loaded yet
   cudaFuncAttributes a;
-  cudaError_t e = cudaFuncGetAttributes(&a, move_kernel<kPack, KVX_LAYOUT_HND>);
-  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, move_kernel<kPack, KVX_LAYOUT_NHD>);
-  return e;
+  return cudaFuncGetAttributes(&a, kernel_of(kPack));
 }
 
-int move_ctas_per_sm(int dir, int layout) {
-  if (dir == kPack) return layout == KVX_LAYOUT_HND ? occupancy_of<kPack, KVX_LAYOUT_HND>()
-                                                    : occupancy_of<kPack, KVX_LAYOUT_NHD>();
-  return layout == KVX_LAYOUT_HND ? occupancy_of<kUnpack, KVX_LAYOUT_HND>()
-                                  : occupancy_of<kUnpack, KVX_LAYOUT_NHD>();
+int move_ctas_per_sm(int dir) {
+  int n = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel_of(dir), kThreads, 0) != cudaSuccess) {
+    cudaGetLastError();
+    return 1;
+  }
+  return n > 0 ? n : 1;
 }
 
 }  // namespace kvx

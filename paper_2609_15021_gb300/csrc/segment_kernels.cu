@@ -28,7 +28,7 @@ __global__ void __launch_bounds__(kThreads) segment_kernel(const __grid_constant
     while (b < b_end) {
       const Segment& S = p.seg[j];
       const int64_t n = min(b_end, S.byte_end) - b;
-      move_flat<kPack>(const_cast<uint8_t*>(S.src) + (b - seg_begin), S.dst + (b - seg_begin), n, lane);
+      copy_flat(S.dst + (b - seg_begin), S.src + (b - seg_begin), n, lane);
       b += n;
       if (b >= S.byte_end && b < b_end) {
         seg_begin = S.byte_end;

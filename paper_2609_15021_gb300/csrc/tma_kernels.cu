@@ -107,7 +107,7 @@ struct Unit {
   uint8_t* pg;   // page side (K or V half of the page)
   uint8_t* ck;   // chunk side
   int nr;        // rows (tokens x heads)
-  int move;      // 0: nothing to move (past a short chunk's end, or a bad page)
+  int move;      // 0: nothing to move (a bad page)
   int full;      // the unit covers the whole page half (all B tokens)
   int layer, kv;
   int page;
@@ -125,21 +125,20 @@ __device__ __forceinline__ Unit decode(const MoveParams& p, int64_t u, int& j, i
   }
   const Job& J = p.jobs[j];
   const int64_t local = u - job_begin;
-  const int kv = (int)(local & 1);
-  const int64_t rest = local >> 1;
-  const int jb = (int)(rest % p.blocks_per_chunk);
-  const int l = J.l0 + (int)(rest / p.blocks_per_chunk);
+  const int64_t plane = local / J.units_per_plane;  // (layer - l0) * 2 + kv
+  const int jb = (int)(local - plane * J.units_per_plane);
+  const int kv = (int)(plane & 1);
+  const int l = J.l0 + (int)(plane >> 1);
   const int tok0 = jb * p.B;
-  if (tok0 >= J.tokens) return r;
   const int nb = min(p.B, J.tokens - tok0);
   const int64_t HR = (int64_t)p.H * p.R;
-  const int64_t kpage = J.first_block + jb;
-  const int64_t lblk = kpage / p.ppb;
+  const uint32_t gp = (uint32_t)J.first_sub + jb, e = gp / (uint32_t)p.ppb;
+  const int64_t lblk = J.first_entry + e;
   const int32_t entry = __ldg(p.table + lblk);
-  const int64_t page = (int64_t)entry * p.ppb + (kpage - lblk * p.ppb);
-  r.ck = J.chunk + ((int64_t)(l - J.l0) * 2 + kv) * J.tokens * HR + (int64_t)tok0 * HR;
+  const int64_t page = (int64_t)entry * p.ppb + (gp - e * p.ppb);
+  r.ck = J.chunk + (plane * J.tokens + tok0) * HR;
   r.nr = nb * p.H;
-  if (entry < 0 || (int64_t)entry >= p.num_blocks / p.ppb) {
+  if ((uint32_t)entry >= p.entries) {
     if (lane == 0) atomicMin(p.err, (long long)lblk);
     if (DIR == kPack && lane >= 0) {
       const uint4 z = make_uint4(0, 0, 0, 0);

@@ -3,8 +3,8 @@
 Sizes are small enough for the oracle to finish in well under a second each,
 yet span several warp units, several kernel launches (more chunks than one
 launch carries), staging batches that split a chunk by layers, ragged last
-pages and short last chunks, a non-zero start, both page layouts, the fast
-(power-of-two row) and generic row paths, and both transfer modes.
+pages and short last chunks, a non-zero start, both page layouts, rows that
+are and are not a power of two, and both transfer modes.
 """
 import numpy as np
 import pytest
@@ -121,6 +121,68 @@ def test_store_load_parity(orc, ctxs, name, mode):
 def test_store_load_parity_staged_tma(orc, ctxs, name):
     """Staged mode with the TMA bulk-copy kernel packing into / unpacking from the ring."""
     _run_case(orc, ctxs(1, 0, kvx().KVX_FLAG_DEVICE_TMA), CASES[name], torch.cuda.Stream())
+
+
+# The load/store kernel's unit is 4 KiB of a plane, one (chunk, layer, K|V), wherever that
+# cuts rows and pages: planes one row short of a unit, of a unit, and one row over; rows longer
+# than a unit; rows and pages that units cut anywhere; pages far smaller than a unit, in logical blocks.
+UNIT_CASES = {
+    "plane_4080B": (2, 600, 1, 1, 8, 2, HND, 511, 255, 0, 0),
+    "plane_4096B": (2, 600, 1, 1, 8, 2, NHD, 513, 256, 0, 0),
+    "plane_4112B": (2, 600, 1, 1, 8, 2, HND, 515, 257, 1, 0),
+    "rows_4112B": (2, 12, 2, 2, 2056, 2, HND, 11, 4, 1, 1),
+    "rows_160B_3_heads": (3, 40, 8, 3, 80, 2, HND, 37, 24, 1, 3),
+    "rows_192B_nhd": (2, 24, 16, 5, 96, 2, NHD, 21, 48, 0, 5),
+    "pages_of_96B_in_logical_blocks": (2, 3 * 90, 1, 3, 16, 1, HND, 83, 30, 1, 0, 3),
+}
+
+
+@pytest.mark.parametrize("mode,flag,max_ctas", [("zerocopy", None, 0), ("zerocopy", None, 1),
+                                                ("staged", "KVX_FLAG_DEVICE_LSU", 0)])
+@pytest.mark.parametrize("name", list(UNIT_CASES))
+def test_load_store_units(orc, ctxs, name, mode, flag, max_ctas):
+    _run_case(orc, ctxs(MODES[mode], 0, getattr(kvx(), flag) if flag else 0, max_ctas), UNIT_CASES[name],
+              torch.cuda.Stream())
+
+
+def test_unit_queues_serve_launch_after_launch(orc):
+    """Launches over the host link of at least eight units a warp take their units from
+    counters that the launch before left at zero (a context keeps 1,280 of them).  With one
+    CTA a 512 KiB transfer does: more launches than counters, on two streams at once, a
+    captured one (which takes no counters) replayed among them, and every byte as it should be."""
+    k = kvx()
+    spec = oracle.PoolSpec(2, 40, 16, 4, 128, 2, HND)
+    T, C = 37 * 16 - 5, 256
+    src_np, table = host_layers(spec, 71), synth.permuted_table(40, 37, 72)
+    want, _ = oracle_store(orc, spec, src_np, table, 0, T, C)
+    poisoned = [np.full(spec.layer_bytes, POISON, np.uint8) for _ in range(2)]
+    want_l, _ = oracle_load(orc, spec, poisoned, table, 0, T, C, want)
+    src, table_d = device_pool(spec, src_np), torch.from_numpy(table).cuda()
+    hosts = [pinned_chunks(orc, spec, 0, T, C) for _ in range(2)]
+    dsts = [device_pool(spec) for _ in range(2)]
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    ctx = k.kv_ctx_create(0, max_ctas=1)
+    try:
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=streams[0]):
+            k.kv_store(ctx, src, table_d, 0, T, C, hosts[0])
+        for i in range(350):
+            for s, host, dst in zip(streams, hosts, dsts):
+                k.kv_store(ctx, src, table_d, 0, T, C, host, stream=s)
+                k.kv_load(ctx, dst, table_d, 0, T, C, host, stream=s)
+            if i % 50 == 0:
+                with torch.cuda.stream(streams[0]):
+                    graph.replay()
+        torch.cuda.synchronize()
+        for host, dst in zip(hosts, dsts):
+            for h, w in zip(host, want):
+                assert first_mismatch(np_of(h), w) is None
+            for l in range(2):
+                assert first_mismatch(np_of(dst.layers[l]), want_l[l]) is None
+        assert k.kv_get_device_error(ctx) == -1
+    finally:
+        k.kv_ctx_destroy(ctx)
 
 
 @pytest.mark.parametrize("name", ["ragged_tail_offset_start", "27b_shape_two_chunks", "fp8_1568_token_chunks"])
