@@ -323,11 +323,13 @@ kvx_status kv_state_load(kvx_ctx* ctx, int32_t num_layers, void* const* layer_ba
  * GPU memory and must not see allocations it does not track, or code that must
  * not let cudaMalloc/cudaFree synchronise the device mid-pipeline.  kv_store
  * needs a context, and a context allocates a staging ring, streams and events.
- * This call creates nothing: it packs into a static device array of
- * KVX_NOALLOC_SCRATCH_BYTES (64 MiB, plus 256 bytes) that every GPU loading
- * this part of the library holds until the process exits, and copies each
- * packed batch to the host chunks with cudaMemcpyAsync, all on `stream` and in
- * stream order (no overlap of packing and copying, unlike kv_store).
+ * This call creates nothing: it writes mapped host chunks directly over the
+ * host link, as kv_store's zero-copy mode does, all on `stream`.  If one of the
+ * chunks is not mapped for the GPU, it packs into a static device array of
+ * KVX_NOALLOC_SCRATCH_BYTES (64 MiB, plus 256 bytes) and copies each packed batch
+ * to the host chunks with cudaMemcpyAsync, in stream order (no overlap of packing
+ * and copying, unlike kv_store).  Every GPU loading this part of the library
+ * holds the array until the process exits.
  *
  * Arguments, layout, alignment, pinned-memory and range rules are those of
  * kv_store; it runs on the calling thread's current device.  One layer of one

@@ -105,11 +105,14 @@ enum Where : int { kHostChunks = 0, kDeviceChunks = 1 };
 // shape and memory, token range, block table, and every chunk pointer of
 // [t0, t1) on `device`.  Fills *g and *n (chunks in the range) and, when
 // `side` is not null, side[i] = the address of chunk i that the kernel or
-// copy engine uses (mapped address for zero-copy host chunks).  Enqueues
+// copy engine uses (mapped address for zero-copy host chunks).  *all_mapped,
+// when not null, tells whether the GPU can reach every host chunk.  Enqueues
 // nothing and allocates nothing.
 kvx_status check_transfer(int device, const kvx_pool* P, const int32_t* table, int64_t table_len, int64_t t0,
                           int64_t t1, int32_t C, void* const* chunks, int64_t n_chunks, cudaStream_t stream,
-                          int where, int mode, Geometry* g, int64_t* n, uint8_t** side);
+                          int where, int mode, Geometry* g, int64_t* n, uint8_t** side, bool* all_mapped = nullptr);
+// Device-side address of page-locked host memory that check_transfer found mapped.
+uint8_t* mapped_address(const void* host);
 void init_params(MoveParams* p, long long* err, const kvx_pool* P, const Geometry& g, const int32_t* table);
 void push_job(MoveParams* p, uint8_t* chunk_side, int64_t first_page, int32_t tokens, int32_t l0, int32_t nl);
 // Cuts the jobs of `p` into units for launch_move; returns the CTAs that give

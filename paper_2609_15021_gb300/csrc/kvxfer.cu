@@ -639,7 +639,7 @@ void set_error_text(const char* text) { snprintf(g_last_error_text, sizeof(g_las
 
 kvx_status check_transfer(int device, const kvx_pool* P, const int32_t* table, int64_t table_len, int64_t t0,
                           int64_t t1, int32_t C, void* const* chunks, int64_t n_chunks, cudaStream_t stream,
-                          int where, int mode, Geometry* g, int64_t* n_out, uint8_t** side) {
+                          int where, int mode, Geometry* g, int64_t* n_out, uint8_t** side, bool* all_mapped) {
   kvx_status st = check_pool_shape(P, g);
   if (st != KVX_OK) return st;
   int64_t n = 0;
@@ -649,6 +649,7 @@ kvx_status check_transfer(int device, const kvx_pool* P, const int32_t* table, i
   st = check_stream_device(stream, device);
   if (st != KVX_OK) return st;
   *n_out = n;
+  if (all_mapped) *all_mapped = true;
   if (n == 0) return KVX_OK;  // empty range: nothing to order or move
   st = check_pool_memory(device, P, *g);
   if (st != KVX_OK) return st;
@@ -672,6 +673,7 @@ kvx_status check_transfer(int device, const kvx_pool* P, const int32_t* table, i
       uint8_t* mapped = nullptr;
       st = check_pinned_range(c, bytes, &mapped);
       if (st != KVX_OK) return st;
+      if (all_mapped && !mapped) *all_mapped = false;
       if (mode == KVX_MODE_ZEROCOPY) {
         if (!mapped) return KVX_ENOTPINNED;
         s = mapped;
@@ -680,6 +682,15 @@ kvx_status check_transfer(int device, const kvx_pool* P, const int32_t* table, i
     if (side) side[i] = s;
   }
   return KVX_OK;
+}
+
+uint8_t* mapped_address(const void* host) {
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, host) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  return (uint8_t*)a.devicePointer;
 }
 
 void init_params(MoveParams* p, long long* err, const kvx_pool* P, const Geometry& g, const int32_t* table) {

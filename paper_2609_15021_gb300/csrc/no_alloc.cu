@@ -1,15 +1,17 @@
-// no_alloc.cu -- kv_store_noalloc: the staged store with its staging buffer in
-// a static device array instead of memory the library allocates.
+// no_alloc.cu -- kv_store_noalloc: the store without a context, written straight
+// to the host chunks or, where the GPU cannot reach one of them, staged in a
+// static device array instead of memory the library allocates.
 //
 // Some callers cannot call cudaMalloc: an engine whose memory pool owns all
 // of the GPU's free memory and must not see allocations it does not track, or
 // code that must not let cudaMalloc / cudaFree synchronise the device in the
 // middle of a pipeline.  They keep inputs and outputs in their own buffers,
-// but the staged store also needs scratch memory to pack chunks before the
-// copy engines move them to the host.  This entry point takes that scratch
-// from g_scratch, a file-scope array of fixed size that every GPU which loads
-// this part of the library holds until the process exits.  It creates no
-// context, stream or event, and allocates no device, pinned or heap memory.
+// but a staged store also needs scratch memory to pack chunks before the copy
+// engines move them to the host, and every store an error word.  This entry
+// point takes that scratch from g_scratch, a file-scope array of fixed size that
+// every GPU which loads this part of the library holds until the process exits.
+// It creates no context, stream or event, and allocates no device, pinned or
+// heap memory.
 //
 // In host code g_scratch is only a host-side stand-in for the symbol, not a
 // device address: it must not be passed to a kernel.  The device address is
@@ -138,8 +140,9 @@ extern "C" kvx_status kv_store_noalloc(const kvx_pool* pool, const int32_t* bloc
     if (st != KVX_OK) return st;
     Geometry g;
     int64_t n = 0;
+    bool mapped = false;
     st = check_transfer(device, pool, block_table, table_len, tok_begin, tok_end, chunk_tokens, host_chunks,
-                        n_chunks, stream, kHostChunks, KVX_MODE_STAGED, &g, &n, nullptr);
+                        n_chunks, stream, kHostChunks, KVX_MODE_STAGED, &g, &n, nullptr, &mapped);
     if (st != KVX_OK || n == 0) return st;
     const int64_t layer_bytes_max =
         2ll * std::min<int64_t>(chunk_tokens, tok_end - tok_begin) * pool->num_heads * g.row;
@@ -161,12 +164,38 @@ extern "C" kvx_status kv_store_noalloc(const kvx_pool* pool, const int32_t* bloc
     }
     uint8_t* staging = base + kSink;
     long long* err = dev_first_bad_block ? (long long*)dev_first_bad_block : (long long*)base;
-
-    // Batches of (chunk, layer range) pieces that fit the array, each packed and
-    // then copied out on the caller's stream.  Stream order alone keeps a batch
-    // from overwriting the array before the previous batch's copies have read it.
     const int64_t first_chunk = tok_begin / chunk_tokens;
     const int64_t bpc = chunk_tokens / pool->block_tokens;
+    auto tokens_of = [&](int64_t i) {
+      return (int32_t)std::min<int64_t>(chunk_tokens, tok_end - (first_chunk + i) * chunk_tokens);
+    };
+
+    // Chunks that the GPU can reach are written by the kernel itself, as kv_store's
+    // zero-copy mode does.  2,048 tokens of a 62-layer pool with 8 heads of 256-byte
+    // rows (520 MB) take 2,695 us; packed and copied batch by batch they took 2,923,
+    // since a batch's packing waits for the copies of the one before (link: 2,688).
+    if (mapped) {
+      int sms = 0;
+      e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+      if (e != cudaSuccess) return fail_cuda(e, "cudaDeviceGetAttribute");
+      MoveParams p;
+      init_params(&p, err, pool, g, block_table);
+      for (int64_t i = 0; i < n; ++i) {
+        uint8_t* chunk = mapped_address(host_chunks[i]);
+        if (!chunk) return KVX_ENOTPINNED;
+        push_job(&p, chunk, (first_chunk + i) * bpc, tokens_of(i), 0, pool->num_layers);
+        if (p.n_jobs < kMaxJobs && i < n - 1) continue;
+        const int64_t grid = std::min<int64_t>(cut_units(&p, true), std::max(1, (sms + 1) / 2));
+        const cudaError_t le = launch_move(kPack, p, (int)grid, stream);
+        if (le != cudaSuccess) return fail_cuda(le, "pack kernel launch");
+        p.n_jobs = 0;
+      }
+      return KVX_OK;
+    }
+
+    // Otherwise batches of (chunk, layer range) pieces that fit the array, each
+    // packed and then copied out on the caller's stream.  Stream order alone keeps a
+    // batch from overwriting the array before the previous batch's copies have read it.
     struct Piece {
       int64_t i;
       int32_t l0, nl;
@@ -174,9 +203,6 @@ extern "C" kvx_status kv_store_noalloc(const kvx_pool* pool, const int32_t* bloc
     } batch[kMaxJobs];
     int nb = 0;
     int64_t used = 0;
-    auto tokens_of = [&](int64_t i) {
-      return std::min<int64_t>(chunk_tokens, tok_end - (first_chunk + i) * chunk_tokens);
-    };
     auto layer_bytes = [&](int64_t i) { return 2ll * tokens_of(i) * pool->num_heads * g.row; };
     auto flush = [&]() -> kvx_status {
       if (nb == 0) return KVX_OK;
@@ -184,7 +210,7 @@ extern "C" kvx_status kv_store_noalloc(const kvx_pool* pool, const int32_t* bloc
       init_params(&p, err, pool, g, block_table);
       int64_t off = 0;
       for (int q = 0; q < nb; ++q) {
-        push_job(&p, staging + off, (first_chunk + batch[q].i) * bpc, (int32_t)tokens_of(batch[q].i), batch[q].l0,
+        push_job(&p, staging + off, (first_chunk + batch[q].i) * bpc, tokens_of(batch[q].i), batch[q].l0,
                  batch[q].nl);
         off += batch[q].bytes;
       }

@@ -568,3 +568,23 @@ def test_chunk_lists_move_what_lists_move(orc, ctxs, mode):
         assert first_mismatch(np_of(dst.layers[l]), want_l[l]) is None, ("load", l)
         assert first_mismatch(np_of(dst2.layers[l]), want_l[l]) is None, ("unpack", l)
     assert k.kv_get_device_error(ctx) == -1
+
+
+@pytest.mark.parametrize("n_chunks,short", [(1, 31), (1, 0), (64, 5), (65, 0), (65, 31), (130, 7)])
+def test_noalloc_launches_of_64_chunks(orc, n_chunks, short):
+    """kv_store_noalloc writes mapped chunks with one launch for every 64 of them: one chunk
+    (of one token, too), a full launch, one chunk over it and three launches."""
+    k = kvx()
+    C = 32
+    spec = oracle.PoolSpec(2, 290, 16, 3, 40, 2, HND)
+    src_np, table = host_layers(spec, 61), synth.permuted_table(290, 2 * n_chunks, 62)
+    T = n_chunks * C - short
+    host = pinned_chunks(orc, spec, 0, T, C, extra=16)
+    k.kv_store_noalloc(device_pool(spec, src_np), torch.from_numpy(table).cuda(), 0, T, C, host)
+    torch.cuda.synchronize()
+    want, _ = oracle_store(orc, spec, src_np, table, 0, T, C)
+    assert len(want) == n_chunks
+    for h, w in zip(host, want):
+        got = np_of(h)
+        assert first_mismatch(got[:-16], w) is None
+        assert np.all(got[-16:] == POISON)
