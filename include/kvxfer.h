@@ -108,13 +108,14 @@ typedef enum {
                                       paper's missing dependency (Sec. 3.2).
                                       Results are then undefined.             */
 /* Device-side moves (kv_pack, kv_unpack, staged mode) use, by default, the
-   TMA kernel when a K or V page half is at most 48 KiB: one tensor-map box
-   per page half for HND pools, one bulk copy per side for NHD pools (whose
-   page halves are contiguous), staged through shared memory; both measured
-   faster than the load/store kernel on GB300.  HND pools that no tensor map
-   describes use the 16-byte load/store kernel.  Zero-copy moves always use
-   the load/store kernel.  The flags below force one of them for device-side
-   moves.                                                                     */
+   TMA kernel when a K or V page half is 8 to 48 KiB: one bulk copy per side where
+   the page half holds its rows in the chunk's order (NHD pools, one head), one
+   tensor-map box per page half for other HND pools, in launches of at least 4 MiB;
+   both staged through shared memory, and measured as fast as the load/store
+   kernel or faster on GB300.  Other page halves, smaller HND launches and HND
+   pools that no tensor map describes use the 16-byte load/store kernel.
+   Zero-copy moves always use the load/store kernel.  The flags below force one of
+   them for device-side moves.                                                */
 #define KVX_FLAG_DEVICE_TMA 0x4u   /* TMA everywhere it fits, with one bulk
                                       copy per row of HND pages no tensor map
                                       describes                              */

@@ -367,15 +367,28 @@ kvx_status launch_move_timed(kvx_ctx* ctx, const kvx_pool* P, int dir, int layou
   // largest unit) of at most 48 KiB: one shared-memory stage per unit, or a
   // ring of 2-3 when a capped grid strides over units.
   // Default: tensor maps for HND pools the TMA unit can describe; one bulk
-  // copy per side for NHD pools, whose units are contiguous on both sides
-  // (measured on GB300 at 32k tokens: 6.95 / 7.00 TB/s against 6.78 / 6.75
-  // with loads/stores); loads/stores otherwise (per-row bulk copies of HND
-  // pages without tensor maps are slower).
+  // copy per side where a half page holds its rows in the chunk's order (NHD
+  // pools, one head, one token); loads/stores otherwise (per-row bulk copies of
+  // HND pages without tensor maps are slower).  Measured on GB300 (us, TMA
+  // against loads/stores, pack and unpack of 16-token bf16 pages):
+  //   half pages of 8 KiB or more, 1 GB: HND 32 KiB 301 / 297 against 302 / 298,
+  //     8 KiB 312 / 306 against 312 / 314; NHD 32 KiB 300 / 296 against 300 / 296
+  //   half pages of 4 KiB, 1 GB: 357 / 355 against 324 / 329; of 2 KiB 627 / 619
+  //     against 350 / 354: a CTA for each is too little work for its launch, so
+  //     half pages below 8 KiB take loads/stores
+  //   HND in replayed graphs, 0.25 / 1 / 2 MB: 3.2 / 4.7 / 6.8 against 2.6 / 3.2 /
+  //     3.3, as a CTA's one box comes in row by row, so launches below 4 MiB take
+  //     loads/stores (8 MB 6.7 against 4.3, 16 MB equal; from 4 MiB on pools of
+  //     such half pages have always had the TMA engine's bounded waits and keep
+  //     them); NHD 2.8 / 3.0 / 3.3, no slower than loads/stores
+  constexpr int64_t kTmaHalf = 8 << 10, kTmaBoxes = 4 << 20;
   const int64_t unit_bytes = (int64_t)p.B * p.H * p.R;
   const uint32_t f = ctx->opts.flags;
-  const bool fits = !over_link && unit_bytes <= (48 << 10) && !(f & KVX_FLAG_DEVICE_LSU);
-  const void* maps = fits && layout == KVX_LAYOUT_HND ? tensor_maps_of(ctx, P, p.R) : nullptr;
-  const bool tma = fits && (maps || layout == KVX_LAYOUT_NHD || (f & KVX_FLAG_DEVICE_TMA));
+  const bool flat = layout == KVX_LAYOUT_NHD || p.H == 1 || p.B == 1;
+  const bool fits = !over_link && unit_bytes <= (48 << 10) && !(f & KVX_FLAG_DEVICE_LSU) &&
+                    ((f & KVX_FLAG_DEVICE_TMA) || (unit_bytes >= kTmaHalf && (flat || bytes >= kTmaBoxes)));
+  const void* maps = fits && !flat ? tensor_maps_of(ctx, P, p.R) : nullptr;
+  const bool tma = fits && (maps || flat || (f & KVX_FLAG_DEVICE_TMA));
   // Grid: HBM-bound launches give every unit its own warp (LSU) or CTA (TMA)
   // and let the block scheduler spread them; measured on GB300 this keeps
   // DRAM busier than a persistent grid walking the units in lockstep.
@@ -412,7 +425,7 @@ kvx_status launch_move_timed(kvx_ctx* ctx, const kvx_pool* P, int dir, int layou
   if (maps)
     KVX_CUDA_AT("launch", launch_move_tmap(dir, p, maps, P->num_layers, (int)grid, stage_bytes, stages, wt, s));
   else if (tma)
-    KVX_CUDA_AT("launch", launch_move_tma(dir, layout, p, (int)grid, stage_bytes, stages, wt, s));
+    KVX_CUDA_AT("launch", launch_move_tma(dir, flat ? KVX_LAYOUT_NHD : KVX_LAYOUT_HND, p, (int)grid, stage_bytes, stages, wt, s));
   else
     KVX_CUDA_AT("launch", launch_move(dir, p, (int)grid, s));
   if (queue) {

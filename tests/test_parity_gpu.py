@@ -588,3 +588,30 @@ def test_noalloc_launches_of_64_chunks(orc, n_chunks, short):
         got = np_of(h)
         assert first_mismatch(got[:-16], w) is None
         assert np.all(got[-16:] == POISON)
+
+
+# Where device-side moves change engine: page halves of 8 KiB less a row, of 8 and of 48 KiB and a
+# row more; HND launches just below, at and above 4 MiB; one head and one token per page (whose
+# halves are copied as they lie), with a ragged end.
+@pytest.mark.parametrize("L,N,B,H,D,e,layout,n_used,C,short", [
+    (2, 40, 15, 2, 128, 2, HND, 37, 60, 7), (2, 40, 16, 2, 128, 2, HND, 37, 64, 7), (2, 40, 16, 2, 128, 2, NHD, 37, 64, 7),
+    (1, 20, 64, 3, 128, 2, HND, 18, 128, 9), (1, 20, 64, 3, 128, 2, NHD, 18, 128, 9), (1, 20, 65, 3, 128, 2, HND, 18, 130, 9),
+    (2, 40, 16, 8, 128, 2, HND, 32, 256, 1), (2, 40, 16, 8, 128, 2, HND, 32, 256, 0), (2, 40, 16, 8, 128, 2, HND, 33, 256, 15),
+    (3, 40, 32, 1, 256, 2, HND, 37, 64, 5), (3, 40, 1, 40, 128, 2, HND, 37, 4, 0)])
+def test_device_engine_borders(orc, ctxs, L, N, B, H, D, e, layout, n_used, C, short):
+    k = kvx()
+    spec = oracle.PoolSpec(L, N, B, H, D, e, layout)
+    src_np, T = host_layers(spec, 91), n_used * B - short
+    ta, tb = synth.permuted_table(N, n_used, 92), synth.permuted_table(N, n_used, 93)
+    want, _ = oracle_store(orc, spec, src_np, ta, 0, T, C)
+    want_l, _ = oracle_load(orc, spec, [np.full(spec.layer_bytes, POISON, np.uint8) for _ in range(L)], tb, 0, T, C, want)
+    ctx, dev, dst = ctxs(2), device_chunks(orc, spec, 0, T, C, extra=16), device_pool(spec)
+    k.kv_pack(ctx, device_pool(spec, src_np), torch.from_numpy(ta).cuda(), 0, T, C, dev)
+    k.kv_unpack(ctx, dst, torch.from_numpy(tb).cuda(), 0, T, C, dev)
+    torch.cuda.synchronize()
+    for d, w in zip(dev, want):
+        got = np_of(d)
+        assert first_mismatch(got[:-16], w) is None and np.all(got[-16:] == POISON)
+    for l in range(L):
+        assert first_mismatch(np_of(dst.layers[l]), want_l[l]) is None, l
+    assert k.kv_get_device_error(ctx) == -1
