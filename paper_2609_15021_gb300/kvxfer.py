@@ -13,6 +13,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import sys
 from dataclasses import dataclass
 from typing import Sequence
 
@@ -223,6 +224,7 @@ class KvPool:
         self._c = kvx_pool(len(self.layers), ctypes.cast(self._bases, ctypes.POINTER(ctypes.c_void_p)),
                            self.num_blocks, self.block_tokens, self.num_heads, self.head_dim,
                            self.elem_bytes, self.layout, self.pages_per_block)
+        self._token_bytes = len(self.layers) * 2 * self.num_heads * self.row_bytes  # of a chunk
 
     @classmethod
     def from_tensors(cls, layers, num_heads: int, block_tokens: int, layout: int = KVX_LAYOUT_HND,
@@ -294,8 +296,9 @@ class ChunkList:
     again over the same chunks.  kv_store / kv_load / kv_pack / kv_unpack /
     kv_store_noalloc take it wherever they take a list of chunks; element i is
     the call's i-th chunk, as in a list, and a slice is a ChunkList over a run
-    of the same chunks, sharing the marshalled addresses.  Per call only the
-    sizes the range needs are compared (vectorised).  The chunks must keep
+    of the same chunks, sharing the marshalled addresses.  Per call the
+    smallest and the last size are compared with what the range needs, and only
+    if one falls short every chunk's.  The chunks must keep
     their storage while the list is in use (it holds references to them)."""
 
     def __init__(self, chunks, nbytes: int | None = None, *, _parent=None, _start=0, _stop=None, _array=None):
@@ -304,7 +307,7 @@ class ChunkList:
         import numpy as np
         if _parent is not None:
             self._items, self._arr, self._sizes = _parent._items, _parent._arr, _parent._sizes
-            self._start, self._n = _start, _stop - _start
+            self._set_run(_start, _stop - _start)
             return
         if _array is not None:  # a ctypes address array the library filled in (tier slots)
             self._arr, n = _array, len(chunks)
@@ -314,12 +317,28 @@ class ChunkList:
             n = len(self._items)
             self._arr = (ctypes.c_void_p * max(1, n))(*[_ptr(c) for c in self._items])
         unknown = np.iinfo(np.int64).max
-        sizes = np.full(n, unknown if nbytes is None else nbytes, dtype=np.int64)
-        for i, c in enumerate(self._items):
-            if not isinstance(c, int):
-                _check_tensor(c, f"chunk {i}")
-                sizes[i] = _nbytes(c)
-        self._sizes, self._start, self._n = sizes, 0, n
+        size = unknown if nbytes is None else nbytes
+        self._sizes = sizes = np.full(n, size, dtype=np.int64)
+        same = _array is not None  # slots of one tier
+        if not same:
+            for i, c in enumerate(self._items):
+                if not isinstance(c, int):
+                    _check_tensor(c, f"chunk {i}")
+                    sizes[i] = _nbytes(c)
+        self._set_run(0, n, size if same else None)
+
+    def _set_run(self, start: int, n: int, size: int | None = None) -> None:
+        """size: every chunk's, if known to be the same."""
+        self._start, self._n = start, n
+        self._ptr = ctypes.cast(ctypes.byref(self._arr, start * ctypes.sizeof(ctypes.c_void_p)),
+                                ctypes.POINTER(ctypes.c_void_p))
+        # the smallest chunk but the last one, which may be a short one, and the last
+        if size is not None:
+            self._least = self._last = size
+            return
+        sizes = self._sizes[start:start + n]
+        self._least = int(sizes[:-1].min()) if n > 1 else sys.maxsize
+        self._last = int(sizes[-1]) if n else sys.maxsize
 
     def __len__(self) -> int:
         return self._n
@@ -335,18 +354,19 @@ class ChunkList:
         return self._items[self._start + key % self._n]
 
     def _pointer(self):
-        return ctypes.cast(ctypes.byref(self._arr, self._start * ctypes.sizeof(ctypes.c_void_p)),
-                           ctypes.POINTER(ctypes.c_void_p))
+        return self._ptr
 
     def _check_sizes(self, per_token: int, chunk_tokens: int, tok_begin: int, tok_end: int) -> None:
-        import numpy as np
         first = tok_begin // chunk_tokens
         used = min(self._n, -(-tok_end // chunk_tokens) - first)
         if used <= 0:
             return
+        short = per_token * min(chunk_tokens, tok_end - (first + used - 1) * chunk_tokens)
+        if self._least >= per_token * chunk_tokens and (self._last if used == self._n else self._least) >= short:
+            return
+        import numpy as np
         need = np.full(used, per_token * chunk_tokens, dtype=np.int64)
-        last = first + used - 1
-        need[-1] = per_token * min(chunk_tokens, tok_end - last * chunk_tokens)
+        need[-1] = short
         sizes = self._sizes[self._start:self._start + used]
         bad = np.nonzero(sizes < need)[0]
         if bad.size:
@@ -371,7 +391,7 @@ def _check_transfer_tensors(pool: KvPool, block_table, tok_begin, tok_end, chunk
     if chunk_tokens < 1 or tok_end <= tok_begin:
         return
     first = tok_begin // chunk_tokens
-    per_token = pool.c.num_layers * 2 * pool.num_heads * pool.row_bytes
+    per_token = pool._token_bytes
     if isinstance(chunks, ChunkList):
         chunks._check_sizes(per_token, chunk_tokens, tok_begin, tok_end)
         return

@@ -175,3 +175,72 @@ def test_modes_pool_info_and_foreign_pointers(orc):
         assert int(d[0]) == 7
     finally:
         buf.close()
+
+
+def test_layers_across_mappings_and_past_them(orc):
+    """Layers are checked one allocation at a time: several in one cudaMalloc allocation; one that
+    spans two mappings of reserved addresses (its whole range is device memory: accepted, moved
+    bit-exactly); one that runs from the second mapping into addresses nothing is mapped to (refused,
+    although the reservation goes on)."""
+    import ctypes
+
+    k = kvx()
+    cu = ctypes.CDLL("libcuda.so.1")
+    u64, size_t = ctypes.c_uint64, ctypes.c_size_t
+    one = torch.from_numpy(np.concatenate(host_layers(SPEC, 77))).cuda()  # both layers in one tensor
+    src_np = host_layers(SPEC, 77)
+    table = synth.permuted_table(SPEC.num_blocks, T // SPEC.block_tokens, 5)
+    tab = torch.from_numpy(table).cuda()
+    want, _ = oracle_store(orc, SPEC, src_np, table, 0, T, C)
+    shape = (SPEC.num_blocks, SPEC.block_tokens, SPEC.num_heads, SPEC.head_dim, SPEC.elem_bytes)
+    n = SPEC.layer_bytes
+
+    class Location(ctypes.Structure):
+        _fields_ = [("type", ctypes.c_int), ("id", ctypes.c_int)]
+
+    class Properties(ctypes.Structure):
+        _fields_ = [("type", ctypes.c_int), ("handles", ctypes.c_int), ("location", Location),
+                    ("win32", ctypes.c_void_p), ("flags", ctypes.c_ubyte * 32)]
+
+    class Access(ctypes.Structure):
+        _fields_ = [("location", Location), ("flags", ctypes.c_int)]
+
+    def ok(rc):
+        assert rc == 0, f"CUresult {rc}"
+
+    gpu = Location(1, 0)
+    props, rw = Properties(type=1, location=gpu), Access(gpu, 3)
+    gran = size_t()
+    ok(cu.cuMemGetAllocationGranularity(ctypes.byref(gran), ctypes.byref(props), 0))
+    m = max(gran.value, 2 << 20)
+    va, mapped = u64(), []
+    ok(cu.cuMemAddressReserve(ctypes.byref(va), size_t(4 * m), size_t(0), u64(0), u64(0)))
+    ctx = k.kv_ctx_create(0)
+    try:
+        for i in range(2):
+            h = u64()
+            ok(cu.cuMemCreate(ctypes.byref(h), size_t(m), ctypes.byref(props), u64(0)))
+            mapped.append(h)
+            ok(cu.cuMemMap(u64(va.value + i * m), size_t(m), size_t(0), h, u64(0)))
+        ok(cu.cuMemSetAccess(va, size_t(2 * m), ctypes.byref(rw), size_t(1)))
+        at = [va.value, va.value + m - n // 2]  # the second one spans both mappings
+        for d, a in zip(at, src_np):
+            ok(cu.cuMemcpyHtoD_v2(u64(d), a.ctypes.data_as(ctypes.c_void_p), size_t(n)))
+        for layers in ([one.data_ptr(), one.data_ptr() + n], at):
+            host = pinned_chunks(orc, SPEC, 0, T, C)
+            k.kv_store(ctx, k.KvPool(layers, *shape), tab, 0, T, C, host)
+            torch.cuda.synchronize()
+            for h, w in zip(host, want):
+                assert first_mismatch(np_of(h), w) is None
+        past = k.KvPool([va.value, va.value + 2 * m - n // 2], *shape)
+        for fn in (k.kv_store, k.kv_load):
+            _rejects(k, k.KVX_EDEVICE, fn, ctx, past, tab, 0, T, C, host)
+        for h, w in zip(host, want):
+            assert first_mismatch(np_of(h), w) is None
+    finally:
+        torch.cuda.synchronize()
+        k.kv_ctx_destroy(ctx)
+        for i, h in enumerate(mapped):
+            cu.cuMemUnmap(u64(va.value + i * m), size_t(m))
+            cu.cuMemRelease(h)
+        cu.cuMemAddressFree(va, size_t(4 * m))
