@@ -116,8 +116,9 @@ uint8_t* mapped_address(const void* host);
 void init_params(MoveParams* p, long long* err, const kvx_pool* P, const Geometry& g, const int32_t* table);
 void push_job(MoveParams* p, uint8_t* chunk_side, int64_t first_page, int32_t tokens, int32_t l0, int32_t nl);
 // Cuts the jobs of `p` into units for launch_move; returns the CTAs that give
-// every unit a warp of its own.  link: the chunks are mapped host memory.
-int64_t cut_units(MoveParams* p, bool link);
+// every unit a warp of its own.  link: the chunks are mapped host memory;
+// queue_warps: the warps that take the units from a queue, 0 without one.
+int64_t cut_units(MoveParams* p, bool link, int64_t queue_warps);
 int64_t chunk_bytes(const kvx_pool* P, const Geometry& g, int64_t tokens);
 void set_error_text(const char* text);
 

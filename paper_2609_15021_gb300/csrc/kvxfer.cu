@@ -101,8 +101,8 @@ constexpr int32_t kDefaultSlots = 4;
 constexpr int64_t kDefaultSlotBytes = 128ll << 20;
 constexpr long long kNoError = LLONG_MAX;
 // Launches over the host link take their units from a queue (UnitQueue) from
-// this many units a warp on; below it warps hardly drift apart.
-constexpr int64_t kQueueRounds = 8;
+// this many bytes a warp on, eight units; below it warps hardly drift apart.
+constexpr int64_t kQueueBytes = 32 << 10;
 // More than the launches the driver lets a host thread run ahead by (1024).
 constexpr uint32_t kUnitQueues = 1280;
 
@@ -439,9 +439,9 @@ kvx_status launch_move_timed(kvx_ctx* ctx, const kvx_pool* P, int dir, int layou
     cap = ctx->opts.max_ctas;
   else if (over_link)
     cap = std::min<int64_t>(ctx->link_ctas, (int64_t)ctx->num_sms * ctx->move_occ[dir]);
-  const int64_t wanted = tma ? cut_pages(&p) : cut_units(&p, over_link);
+  UnitQueue* queue = over_link && bytes >= kQueueBytes * cap * (kThreads / 32) ? take_unit_queue(ctx, s) : nullptr;
+  const int64_t wanted = tma ? cut_pages(&p) : cut_units(&p, over_link, queue ? cap * (kThreads / 32) : 0);
   const int64_t grid = std::max<int64_t>(1, std::min(wanted, cap));
-  UnitQueue* queue = over_link && wanted >= kQueueRounds * grid ? take_unit_queue(ctx, s) : nullptr;
   p.units = queue ? *queue : UnitQueue{};
   p.units.ticket++;
   int stage_bytes = 0, stages = 0;

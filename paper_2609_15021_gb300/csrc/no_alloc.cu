@@ -185,7 +185,7 @@ extern "C" kvx_status kv_store_noalloc(const kvx_pool* pool, const int32_t* bloc
         if (!chunk) return KVX_ENOTPINNED;
         push_job(&p, chunk, (first_chunk + i) * bpc, tokens_of(i), 0, pool->num_layers);
         if (p.n_jobs < kMaxJobs && i < n - 1) continue;
-        const int64_t grid = std::min<int64_t>(cut_units(&p, true), std::max(1, (sms + 1) / 2));
+        const int64_t grid = std::min<int64_t>(cut_units(&p, true, 0), std::max(1, (sms + 1) / 2));
         const cudaError_t le = launch_move(kPack, p, (int)grid, stream);
         if (le != cudaSuccess) return fail_cuda(le, "pack kernel launch");
         p.n_jobs = 0;
@@ -215,7 +215,7 @@ extern "C" kvx_status kv_store_noalloc(const kvx_pool* pool, const int32_t* bloc
         off += batch[q].bytes;
       }
       // one warp per unit, as for the library's other HBM-bound launches
-      const int64_t grid = std::max<int64_t>(1, cut_units(&p, false));
+      const int64_t grid = std::max<int64_t>(1, cut_units(&p, false, 0));
       cudaError_t le = launch_move(kPack, p, (int)grid, stream);
       if (le != cudaSuccess) return fail_cuda(le, "pack kernel launch");
       int64_t soff = 0;

@@ -8,8 +8,8 @@
 // load/store units with 16-byte vectors; no tensor cores are involved.
 //
 // Work unit: one batch, 4 KiB of one plane -- one (chunk, layer, K|V) -- handled
-// by one warp, kInflight 16-byte vectors per lane; where HBM bounds a large
-// launch, two batches.  The chunk side of a
+// by one warp, kInflight 16-byte vectors per lane; in large launches a few
+// batches.  The chunk side of a
 // plane is one contiguous extent in [token][head][row] order, so a unit is
 // contiguous there whatever the page and row sizes are, and its vectors are
 // found on the page side ([head][token] order for HND, [token][head] for NHD)
@@ -21,6 +21,8 @@
 // Out-of-range block-table entries skip their vectors (a pack writes zeros)
 // and lower a device error word (atomicMin of the logical block index);
 // nothing traps.
+
+#include <algorithm>
 
 #include "copy16.cuh"
 #include "kvx_internal.h"
@@ -34,6 +36,12 @@ constexpr int kBatchVectors = 32 * kInflight;  // 4 KiB
 // pages with one head of 256-byte rows took 337 us with units of one batch, 322
 // of two, 333 of four; with 8 heads 316, 300 and 306; packing 4 MB 9, 9 and 13 us.
 constexpr int64_t kBatchesApart = 8192;
+// Taken from a queue, a unit is up to 8 batches as long as every warp gets 24
+// units: a 32k-token restore of the 27B shape (8.3 GB) takes 39,377 us with
+// 8, 39,391 with 4, 39,430 with 1 and 39,419 with 32, but 400 MB 2,094 us with 1,
+// 2,097 with 8 and 2,110 with 32 (the last units end apart).
+constexpr int64_t kQueueBatches = 8;
+constexpr int64_t kQueueUnits = 24;
 
 __device__ __forceinline__ uint32_t div_by(uint32_t n, const FastDiv& f) {
   return f.d == 1 ? n : (uint32_t)__umul64hi(f.m, n);
@@ -62,8 +70,8 @@ __device__ __forceinline__ uint64_t div_by(uint64_t n, const FastDiv& f) {
 //     256 MB: 1329 us (1508); one 128-byte head: 1334 us (1455)
 //   pack / unpack in device memory, 1 GB: 300 / 298 us, 6.8 TB/s (308 / 310);
 //     head_dim 96: 304 / 304 us (476 / 451); one 128-byte head: 350 / 354 (606 / 600)
-// Over the link a unit is one batch: units of eight (32 KiB a warp) took 4945 us
-// for the 1 GB restore and 5370 for the store, and equal shares of 26,368 B, so
+// Dealt out in advance over the link a unit is one batch: units of eight took 4945
+// us for the 1 GB restore and 5370 for the store, and equal shares of 26,368 B, so
 // that a warp's last batch is not whole, 95 us for a 16 MB restore instead of 83.
 // 80 registers, 3 CTAs per SM; at 64 it spills 48 bytes, and unpacking 1 GB into
 // HBM takes 310 us.
@@ -149,11 +157,13 @@ MoveKernel kernel_of(int dir) { return dir == kPack ? move_kernel<kPack> : move_
 
 }  // namespace
 
-int64_t cut_units(MoveParams* p, bool link) {
+int64_t cut_units(MoveParams* p, bool link, int64_t queue_warps) {
   const auto vectors = [p](const Job& J) { return (int64_t)J.tokens * p->H * p->by_row.d; };
   int64_t batches = 0;  // of the launch
   for (int32_t i = 0; i < p->n_jobs; ++i) batches += 2ll * p->jobs[i].nl * vectors(p->jobs[i]) / kBatchVectors;
-  p->unit_vectors = (link || batches <= kBatchesApart ? 1 : 2) * kBatchVectors;
+  int64_t per_unit = !link && batches > kBatchesApart ? 2 : 1;
+  if (queue_warps > 0) per_unit = std::max<int64_t>(1, std::min(kQueueBatches, batches / (kQueueUnits * queue_warps)));
+  p->unit_vectors = (uint32_t)(per_unit * kBatchVectors);
   p->total_units = 0;
   for (int32_t i = 0; i < p->n_jobs; ++i) {
     Job& J = p->jobs[i];
