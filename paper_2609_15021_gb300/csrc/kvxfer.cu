@@ -873,18 +873,18 @@ kvx_status state_copy(kvx_ctx* ctx, int32_t L, void* const* layer_base, int64_t 
       s.byte_end = p.total_bytes;
       bytes += slot_bytes;
       if (p.n_seg == kMaxSegments || l == L - 1) {
-        // Warps of at most 32 KiB units, then the unit size that splits the
-        // bytes evenly over those warps in whole rounds: with 32 KiB units a
-        // 48-layer state snapshot took 3 rounds of 608 warps where 2.7 suffice.
-        constexpr int64_t kMaxUnit = 32 << 10, kWarps = kThreads / 32;
+        // Units of one 4 KiB batch, or an even share for every warp where that is
+        // less.  In replayed graphs a 48-layer state snapshot (52.7 MB) restores in
+        // 252 us (256 in three equal units of 29,184 B a warp; link 249) and stores in
+        // 273 (274.5; 272); 4 layers of 64 KiB in 3.5 and 2.4 us (9.0 and 7.2 on the
+        // eight warps that units of 32 KiB make).
+        constexpr int64_t kMaxUnit = 4 << 10, kWarps = kThreads / 32;
         int64_t grid = (p.total_bytes + kMaxUnit * kWarps - 1) / (kMaxUnit * kWarps);
         int64_t cap = (int64_t)ctx->num_sms * ctx->seg_occ;
         cap = std::min<int64_t>(cap, ctx->opts.max_ctas > 0 ? ctx->opts.max_ctas : ctx->link_ctas);
         grid = std::max<int64_t>(1, std::min(grid, cap));
-        const int64_t warps = grid * kWarps;
-        const int64_t rounds = (p.total_bytes + warps * kMaxUnit - 1) / (warps * kMaxUnit);
-        const int64_t share = (p.total_bytes + warps * rounds - 1) / (warps * rounds);
-        p.unit_bytes = std::max<int64_t>(512, (share + 511) / 512 * 512);
+        const int64_t share = (p.total_bytes + grid * kWarps - 1) / (grid * kWarps);
+        p.unit_bytes = std::max<int64_t>(512, std::min(kMaxUnit, (share + 511) / 512 * 512));
         p.total_units = (p.total_bytes + p.unit_bytes - 1) / p.unit_bytes;
         const bool timing = (ctx->opts.flags & KVX_FLAG_TIME_KERNELS) != 0;
         cudaEvent_t a = timing ? take_timing_event(ctx) : nullptr;
