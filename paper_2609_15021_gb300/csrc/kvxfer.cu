@@ -101,7 +101,7 @@ constexpr int32_t kDefaultSlots = 4;
 constexpr int64_t kDefaultSlotBytes = 128ll << 20;
 constexpr long long kNoError = LLONG_MAX;
 // Launches over the host link take their units from a queue (UnitQueue) from
-// this many bytes a warp on, eight units; below it warps hardly drift apart.
+// this many bytes a warp on, eight batches; below it warps hardly drift apart.
 constexpr int64_t kQueueBytes = 32 << 10;
 // More than the launches the driver lets a host thread run ahead by (1024).
 constexpr uint32_t kUnitQueues = 1280;
@@ -415,18 +415,21 @@ kvx_status launch_move_timed(kvx_ctx* ctx, const kvx_pool* P, int dir, int layou
   //     8 KiB 312 / 306 against 312 / 314; NHD 32 KiB 300 / 296 against 300 / 296
   //   half pages of 4 KiB, 1 GB: 357 / 355 against 324 / 329; of 2 KiB 627 / 619
   //     against 350 / 354: a CTA for each is too little work for its launch, so
-  //     half pages below 8 KiB take loads/stores
+  //     half pages below 8 KiB take loads/stores, but flat ones of 4 KiB only
+  //     from 160 MiB on (32 MB 12.9 / 12.9 against 15 / 15, 128 MB 45.7 / 43.6
+  //     against 45.7 / 45.7, 256 MB 88.7 / 88.7 against 82.6 / 84.6)
   //   HND in replayed graphs, 0.25 / 1 / 2 MB: 3.2 / 4.7 / 6.8 against 2.6 / 3.2 /
   //     3.3, as a CTA's one box comes in row by row, so launches below 4 MiB take
   //     loads/stores (8 MB 6.7 against 4.3, 16 MB equal; from 4 MiB on pools of
   //     such half pages have always had the TMA engine's bounded waits and keep
   //     them); NHD 2.8 / 3.0 / 3.3, no slower than loads/stores
-  constexpr int64_t kTmaHalf = 8 << 10, kTmaBoxes = 4 << 20;
+  constexpr int64_t kTmaHalf = 8 << 10, kTmaBoxes = 4 << 20, kFlatHalf = 4 << 10, kFlatMost = 160 << 20;
   const int64_t unit_bytes = (int64_t)p.B * p.H * p.R;
   const uint32_t f = ctx->opts.flags;
   const bool flat = layout == KVX_LAYOUT_NHD || p.H == 1 || p.B == 1;
   const bool fits = !over_link && unit_bytes <= (48 << 10) && !(f & KVX_FLAG_DEVICE_LSU) &&
-                    ((f & KVX_FLAG_DEVICE_TMA) || (unit_bytes >= kTmaHalf && (flat || bytes >= kTmaBoxes)));
+                    ((f & KVX_FLAG_DEVICE_TMA) || (unit_bytes >= kTmaHalf && (flat || bytes >= kTmaBoxes)) ||
+                     (flat && unit_bytes >= kFlatHalf && bytes < kFlatMost));
   const void* maps = fits && !flat ? tensor_maps_of(ctx, P, p.R) : nullptr;
   const bool tma = fits && (maps || flat || (f & KVX_FLAG_DEVICE_TMA));
   // Grid: HBM-bound launches give every unit its own warp (LSU) or CTA (TMA)

@@ -36,12 +36,13 @@ constexpr int kBatchVectors = 32 * kInflight;  // 4 KiB
 // pages with one head of 256-byte rows took 337 us with units of one batch, 322
 // of two, 333 of four; with 8 heads 316, 300 and 306; packing 4 MB 9, 9 and 13 us.
 constexpr int64_t kBatchesApart = 8192;
-// Taken from a queue, a unit is up to 8 batches as long as every warp gets 24
-// units: a 32k-token restore of the 27B shape (8.3 GB) takes 39,377 us with
-// 8, 39,391 with 4, 39,430 with 1 and 39,419 with 32, but 400 MB 2,094 us with 1,
-// 2,097 with 8 and 2,110 with 32 (the last units end apart).
-constexpr int64_t kQueueBatches = 8;
-constexpr int64_t kQueueUnits = 24;
+// Taken from a queue, a unit is up to 4 batches as long as every warp gets 24
+// units, and 8 where every warp gets 64 of these (the last units end apart).  A
+// 32k-token restore of the 27B shape (8.3 GB) takes 39,377 us with 8, 39,391 with
+// 4, 39,430 with 1 and 39,419 with 32; 400 MB 2,095 us with 4, 2,097 with 8 and
+// 2,110 with 32; storing one chunk (65 MB) 342 us with 1, 344 with 4, 346 with 8.
+constexpr int64_t kQueueBatches = 4, kQueueUnits = 24;
+constexpr int64_t kLargeBatches = 8, kLargeUnits = 64;
 
 __device__ __forceinline__ uint32_t div_by(uint32_t n, const FastDiv& f) {
   return f.d == 1 ? n : (uint32_t)__umul64hi(f.m, n);
@@ -162,7 +163,10 @@ int64_t cut_units(MoveParams* p, bool link, int64_t queue_warps) {
   int64_t batches = 0;  // of the launch
   for (int32_t i = 0; i < p->n_jobs; ++i) batches += 2ll * p->jobs[i].nl * vectors(p->jobs[i]) / kBatchVectors;
   int64_t per_unit = !link && batches > kBatchesApart ? 2 : 1;
-  if (queue_warps > 0) per_unit = std::max<int64_t>(1, std::min(kQueueBatches, batches / (kQueueUnits * queue_warps)));
+  if (queue_warps > 0) {
+    per_unit = std::max<int64_t>(1, std::min(kQueueBatches, batches / (kQueueUnits * queue_warps)));
+    if (batches >= kLargeBatches * kLargeUnits * queue_warps) per_unit = kLargeBatches;
+  }
   p->unit_vectors = (uint32_t)(per_unit * kBatchVectors);
   p->total_units = 0;
   for (int32_t i = 0; i < p->n_jobs; ++i) {
