@@ -235,16 +235,23 @@ bool plain_allocation(int device, const void* p, const uint8_t** begin, const ui
 
 // Layers of `bytes` each: 16-byte aligned device memory of `device`.  One query
 // to the driver for every allocation they lie in, where both ends of each
-// layer took two (7.4 us for 62 layers on a Grace core; now 3.6 in allocations
-// of their own, 0.1 in one).
+// layer took two (a call on 62 layers in allocations of their own takes 4.8 us
+// on a Grace core, 14.0 with two queries a layer).  After two layers that lie in
+// no plain allocation, two queries a layer: a pool in virtual memory would pay a
+// third for every layer (30.2 us against 23.1).
 kvx_status check_layers(int device, void* const* base, int32_t layers, int64_t bytes) {
   const uint8_t *begin = nullptr, *end = nullptr;  // the allocation of the layer before
+  int others = 0;  // layers in no plain allocation
   for (int32_t l = 0; l < layers; ++l) {
     const uint8_t* b = (const uint8_t*)base[l];
     if (!b) return KVX_EINVAL;
     if ((uintptr_t)b & 15) return KVX_EALIGN;
     if (b >= begin && b < end && bytes <= end - b) continue;
-    if (plain_allocation(device, b, &begin, &end) && b >= begin && b < end && bytes <= end - b) continue;
+    if (others < 2) {
+      const bool plain = plain_allocation(device, b, &begin, &end);
+      if (plain && b >= begin && b < end && bytes <= end - b) continue;
+      if (!plain) ++others;
+    }
     begin = end = nullptr;
     const kvx_status st = check_device_range(device, b, bytes);
     if (st != KVX_OK) return st;

@@ -7,6 +7,8 @@ cudaPointerGetAttributes, pinned mappings) and the range and alignment rules
 through the same entry points: kv_store, kv_load, kv_pack, kv_unpack,
 kv_state_store, kv_state_load and kv_store_noalloc.
 """
+from dataclasses import replace
+
 import numpy as np
 import pytest
 import torch
@@ -181,7 +183,8 @@ def test_layers_across_mappings_and_past_them(orc):
     """Layers are checked one allocation at a time: several in one cudaMalloc allocation; one that
     spans two mappings of reserved addresses (its whole range is device memory: accepted, moved
     bit-exactly); one that runs from the second mapping into addresses nothing is mapped to (refused,
-    although the reservation goes on)."""
+    although the reservation goes on).  And one layer of each kind, in either order: after two
+    layers outside cudaMalloc's allocations the others are checked by their two ends."""
     import ctypes
 
     k = kvx()
@@ -226,16 +229,23 @@ def test_layers_across_mappings_and_past_them(orc):
         at = [va.value, va.value + m - n // 2]  # the second one spans both mappings
         for d, a in zip(at, src_np):
             ok(cu.cuMemcpyHtoD_v2(u64(d), a.ctypes.data_as(ctypes.c_void_p), size_t(n)))
-        for layers in ([one.data_ptr(), one.data_ptr() + n], at):
-            host = pinned_chunks(orc, SPEC, 0, T, C)
-            k.kv_store(ctx, k.KvPool(layers, *shape), tab, 0, T, C, host)
+        both = [one.data_ptr(), one.data_ptr() + n]
+        # (address, which layer's bytes); the last list runs on past two layers outside plain allocations
+        p0, p1, v0, v1 = (both[0], 0), (both[1], 1), (at[0], 0), (at[1], 1)
+        for layers in ([p0, p1], [v0, v1], [p0, v1], [v0, p1], [v0, p0, v1, v1, p1, v0, p0]):
+            spec = replace(SPEC, num_layers=len(layers))
+            host = pinned_chunks(orc, spec, 0, T, C)
+            k.kv_store(ctx, k.KvPool([a for a, _ in layers], *shape), tab, 0, T, C, host)
             torch.cuda.synchronize()
-            for h, w in zip(host, want):
+            made = [np.concatenate([w.reshape(2, -1)[i] for _, i in layers]) for w in want]
+            for h, w in zip(host, made):
                 assert first_mismatch(np_of(h), w) is None
-        past = k.KvPool([va.value, va.value + 2 * m - n // 2], *shape)
-        for fn in (k.kv_store, k.kv_load):
-            _rejects(k, k.KVX_EDEVICE, fn, ctx, past, tab, 0, T, C, host)
-        for h, w in zip(host, want):
+        end = va.value + 2 * m - n // 2
+        for layers in ([at[0], end], [both[0], end], [at[0], at[1], both[0], end], [at[0], at[1], host[0].data_ptr()]):
+            past = k.KvPool(layers, *shape)
+            for fn in (k.kv_store, k.kv_load):
+                _rejects(k, k.KVX_EDEVICE, fn, ctx, past, tab, 0, T, C, host)
+        for h, w in zip(host, made):
             assert first_mismatch(np_of(h), w) is None
     finally:
         torch.cuda.synchronize()
