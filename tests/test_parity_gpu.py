@@ -145,6 +145,30 @@ def test_load_store_units(orc, ctxs, name, mode, flag, max_ctas):
               torch.cuda.Stream())
 
 
+# Launches over the link whose units come from a queue, with one CTA (eight warps): bytes of the
+# whole range, in 4 KiB batches, where the queue begins (a restore at 32 batches, a store at 64).
+# Rows, pages and planes that batches cut anywhere: rows of 192 B in HND, of 80 B in NHD, one-head
+# pages of 288 B in logical blocks of seven.
+UNIT_SHAPES = {"hnd_192B_rows": (2, 16, 3, 96, 2, HND, 1), "nhd_80B_rows": (2, 8, 5, 40, 2, NHD, 1),
+               "pages_of_288B": (3, 6, 1, 48, 1, HND, 7)}
+
+
+def _batches_case(shape, batches, full):
+    """One chunk of the fewest tokens that fill `batches` batches, or (not full) of one token less."""
+    L, B, H, D, e, layout, ppb = UNIT_SHAPES[shape]
+    T = -(-batches * 4096 // (L * 2 * H * D * e)) - (not full)
+    n_used = -(-T // (B * ppb))
+    C = n_used * B * ppb
+    return (L, (n_used + 3) * ppb, B, H, D, e, layout, n_used, C, 0, C - T, ppb)
+
+
+@pytest.mark.parametrize("full", [False, True])
+@pytest.mark.parametrize("batches", [32, 64])
+@pytest.mark.parametrize("shape", list(UNIT_SHAPES))
+def test_where_the_unit_queue_begins(orc, ctxs, shape, batches, full):
+    _run_case(orc, ctxs(2, 0, 0, 1), _batches_case(shape, batches, full), torch.cuda.Stream())
+
+
 def test_unit_queues_serve_launch_after_launch(orc):
     """Launches over the host link of at least eight units a warp take their units from
     counters that the launch before left at zero (a context keeps 1,280 of them).  With one
