@@ -123,7 +123,7 @@ int64_t chunk_bytes(const kvx_pool* P, const Geometry& g, int64_t tokens);
 void set_error_text(const char* text);
 
 // Launchers (pack_kernels.cu).  Return the cudaError_t of the launch.
-cudaError_t launch_move(int dir, const MoveParams& p, int grid, cudaStream_t s);
+cudaError_t launch_move(int dir, bool link, const MoveParams& p, int grid, cudaStream_t s);
 cudaError_t launch_segments(const SegmentParams& p, int grid, cudaStream_t s);
 // Loads the pack kernels into the current context if lazy loading has not yet.
 cudaError_t load_pack_kernels();
@@ -150,7 +150,7 @@ constexpr int kTensorMapBytes = 128;
 bool encode_tensor_maps(const kvx_pool* P, int64_t row_bytes, void* out);
 cudaError_t launch_move_tmap(int dir, const MoveParams& p, const void* maps, int num_layers, int grid,
                              int stage_bytes, int stages, const TmaWait& wt, cudaStream_t s);
-int move_ctas_per_sm(int dir);
+int link_ctas_per_sm(int dir);
 int segment_ctas_per_sm();
 // Shared tier (tier_kernels.cu): publication of up to kMaxPublish commits in
 // one launch.  Thread j makes a system-scope release store of seq0 + j to the

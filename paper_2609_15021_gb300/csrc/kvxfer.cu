@@ -125,7 +125,7 @@ struct kvx_ctx {
   int32_t store_mode = KVX_MODE_STAGED;
   int32_t load_mode = KVX_MODE_STAGED;
   int num_sms = 1;
-  int move_occ[2] = {1, 1};
+  int move_occ[2] = {1, 1};  // CTAs per SM of the launches that cross the host link
   int seg_occ = 1;
   int link_ctas = 1;  // default CTA cap of launches that cross the host link
   cudaStream_t s_kern = nullptr;  // pack / unpack kernels
@@ -483,7 +483,7 @@ kvx_status launch_move_timed(kvx_ctx* ctx, const kvx_pool* P, int dir, int layou
   else if (tma)
     KVX_CUDA_AT("launch", launch_move_tma(dir, flat ? KVX_LAYOUT_NHD : KVX_LAYOUT_HND, p, (int)grid, stage_bytes, stages, wt, s));
   else
-    KVX_CUDA_AT("launch", launch_move(dir, p, (int)grid, s));
+    KVX_CUDA_AT("launch", launch_move(dir, over_link, p, (int)grid, s));
   if (queue) {
     queue->base += (uint32_t)p.total_units;
     queue->done_base += (uint32_t)grid;
@@ -1078,7 +1078,7 @@ kvx_status kv_ctx_create(int device, const kvx_opts* opts, kvx_ctx** out) {
     ctx->queues.resize(kUnitQueues);
     for (uint32_t i = 0; i < kUnitQueues; ++i)
       ctx->queues[i] = {ctx->d_queues + 2 * i, ctx->queue_done_dev + i, 0, 0, 0};
-    for (int d = 0; d < 2; ++d) ctx->move_occ[d] = move_ctas_per_sm(d);
+    for (int d = 0; d < 2; ++d) ctx->move_occ[d] = link_ctas_per_sm(d);
     ctx->seg_occ = segment_ctas_per_sm();
     if ((e = prepare_tma_kernels()) != cudaSuccess) return fail(e);
     // the host-page touch threads, once per process, at set-up rather than

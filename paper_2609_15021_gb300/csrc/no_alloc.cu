@@ -186,7 +186,7 @@ extern "C" kvx_status kv_store_noalloc(const kvx_pool* pool, const int32_t* bloc
         push_job(&p, chunk, (first_chunk + i) * bpc, tokens_of(i), 0, pool->num_layers);
         if (p.n_jobs < kMaxJobs && i < n - 1) continue;
         const int64_t grid = std::min<int64_t>(cut_units(&p, true, 0), std::max(1, (sms + 1) / 2));
-        const cudaError_t le = launch_move(kPack, p, (int)grid, stream);
+        const cudaError_t le = launch_move(kPack, true, p, (int)grid, stream);
         if (le != cudaSuccess) return fail_cuda(le, "pack kernel launch");
         p.n_jobs = 0;
       }
@@ -216,7 +216,7 @@ extern "C" kvx_status kv_store_noalloc(const kvx_pool* pool, const int32_t* bloc
       }
       // one warp per unit, as for the library's other HBM-bound launches
       const int64_t grid = std::max<int64_t>(1, cut_units(&p, false, 0));
-      cudaError_t le = launch_move(kPack, p, (int)grid, stream);
+      cudaError_t le = launch_move(kPack, false, p, (int)grid, stream);
       if (le != cudaSuccess) return fail_cuda(le, "pack kernel launch");
       int64_t soff = 0;
       for (int q = 0; q < nb;) {

@@ -76,7 +76,16 @@ __device__ __forceinline__ uint64_t div_by(uint64_t n, const FastDiv& f) {
 // that a warp's last batch is not whole, 95 us for a 16 MB restore instead of 83.
 // 80 registers, 3 CTAs per SM; at 64 it spills 48 bytes, and unpacking 1 GB into
 // HBM takes 310 us.
-template <int DIR>
+// LINK, for launches over the host link: the page-side addresses of a batch are
+// all worked out before its data is waited for.  The table entries are then on
+// their way together with a restore's loads from the host, and a store's loads
+// wait for one trip to the table, not for eight: restores of up to 80 MB take 0.5
+// to 1 us less than with the addresses worked out vector by vector (in replayed
+// graphs 4 MB 21.4 us against 22.4), stores 0 to 0.3.  A restore's addresses spill
+// 80 bytes at 80 registers, which costs nothing over the link; with 96 it spills
+// none, but a GEMM beside it keeps 2 to 3 % less of its rate.  In device memory other warps hide the
+// trips, and spilling costs: unpacking 1 GB with one head 333 us against 313.
+template <int DIR, bool LINK>
 __global__ void __launch_bounds__(kThreads, 3) move_kernel(const __grid_constant__ MoveParams p) {
   const uint32_t lane = threadIdx.x & 31;
   const uint32_t nwarps = gridDim.x * (kThreads / 32);
@@ -105,8 +114,10 @@ __global__ void __launch_bounds__(kThreads, 3) move_kernel(const __grid_constant
     uint32_t col = (uint32_t)(first - row * p.by_row.d), h = (uint32_t)(row - tok * p.H);
     uint32_t sp = (uint32_t)tok - page * p.B, e = div_by(gp, p.by_group), sub = gp - e * p.ppb;
     const int32_t* entries = p.table + J.first_entry;
+    uint32_t bad = ~0u;  // lowest entry out of range whose page begins in this lane's vectors
     for (; nv > 0; nv -= kInflight, ck += kInflight * 512) {
       uint4 data[kInflight];
+      uint8_t* page_side[kInflight];  // null: no page to move to or from
       if (DIR == kUnpack) {
 #pragma unroll
         for (int i = 0; i < kInflight; ++i)
@@ -119,14 +130,15 @@ __global__ void __launch_bounds__(kThreads, 3) move_kernel(const __grid_constant
           const bool ok = entry < p.entries;
           const int64_t in_page = (int64_t)(h * p.head_step + sp * p.tok_step) * p.R + col * 16;
           uint8_t* pg = base + ((int64_t)entry * p.ppb + sub) * p.page_bytes + in_page;
-          if (DIR == kPack) {
+          if (LINK) {
+            page_side[i] = ok ? pg : nullptr;
+          } else if (DIR == kPack) {
             data[i] = make_uint4(0, 0, 0, 0);
             if (ok) data[i] = ld16(pg);
           } else if (ok) {
             st16(pg, data[i]);
           }
-          // reported once for each plane, by the page's first vector
-          if (!ok && in_page == 0) atomicMin(p.err, (long long)(J.first_entry + e));
+          bad = !ok && in_page == 0 ? min(bad, e) : bad;
         }
         // 32 vectors on
         col += p.step_col;
@@ -139,12 +151,26 @@ __global__ void __launch_bounds__(kThreads, 3) move_kernel(const __grid_constant
         if (sp >= p.B) sp -= p.B, ++sub;
         if (sub >= p.ppb) sub -= p.ppb, ++e;
       }
+      if (LINK) {
+#pragma unroll
+        for (int i = 0; i < kInflight; ++i) {
+          if (DIR == kPack) data[i] = make_uint4(0, 0, 0, 0);
+          if (i < nv && page_side[i]) {
+            if (DIR == kPack)
+              data[i] = ld16(page_side[i]);
+            else
+              st16(page_side[i], data[i]);
+          }
+        }
+      }
       if (DIR == kPack) {
 #pragma unroll
         for (int i = 0; i < kInflight; ++i)
           if (i < nv) st16(ck + i * 512, data[i]);
       }
     }
+    // reported once for each plane, by the page's first vector
+    if (bad != ~0u) atomicMin(p.err, (long long)(J.first_entry + bad));
     u = nwarps + (p.units.taken ? __shfl_sync(0xffffffffu, next, 0) : u);
   }
   if (!p.units.taken) return;
@@ -154,7 +180,10 @@ __global__ void __launch_bounds__(kThreads, 3) move_kernel(const __grid_constant
 }
 
 using MoveKernel = void (*)(MoveParams);
-MoveKernel kernel_of(int dir) { return dir == kPack ? move_kernel<kPack> : move_kernel<kUnpack>; }
+MoveKernel kernel_of(int dir, bool link) {
+  if (dir == kPack) return link ? move_kernel<kPack, true> : move_kernel<kPack, false>;
+  return link ? move_kernel<kUnpack, true> : move_kernel<kUnpack, false>;
+}
 
 }  // namespace
 
@@ -179,20 +208,21 @@ int64_t cut_units(MoveParams* p, bool link, int64_t queue_warps) {
   return (p->total_units + kWarps - 1) / kWarps;
 }
 
-cudaError_t launch_move(int dir, const MoveParams& p, int grid, cudaStream_t s) {
-  kernel_of(dir)<<<grid, kThreads, 0, s>>>(p);
+cudaError_t launch_move(int dir, bool link, const MoveParams& p, int grid, cudaStream_t s) {
+  kernel_of(dir, link)<<<grid, kThreads, 0, s>>>(p);
   return cudaGetLastError();
 }
 
 cudaError_t load_pack_kernels() {
   // cudaFuncGetAttributes makes CUDA load a kernel that lazy loading has not loaded yet
   cudaFuncAttributes a;
-  return cudaFuncGetAttributes(&a, kernel_of(kPack));
+  const cudaError_t e = cudaFuncGetAttributes(&a, kernel_of(kPack, true));
+  return e == cudaSuccess ? cudaFuncGetAttributes(&a, kernel_of(kPack, false)) : e;
 }
 
-int move_ctas_per_sm(int dir) {
+int link_ctas_per_sm(int dir) {
   int n = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel_of(dir), kThreads, 0) != cudaSuccess) {
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel_of(dir, true), kThreads, 0) != cudaSuccess) {
     cudaGetLastError();
     return 1;
   }

@@ -317,6 +317,40 @@ def test_out_of_range_pages_reported(orc, ctxs, mode):
         assert first_mismatch(np_of(h), w) is None
 
 
+@pytest.mark.parametrize("mode,flag,max_ctas", [("zerocopy", None, 1), ("staged", "KVX_FLAG_DEVICE_LSU", 0)])
+@pytest.mark.parametrize("batches", [60, 800])
+@pytest.mark.parametrize("shape", list(UNIT_SHAPES))
+def test_bad_entries_inside_units(orc, ctxs, shape, batches, mode, flag, max_ctas):
+    """Several bad entries, among them the first, the last, neighbours and the extreme values, in units
+    that span many pages (over the link of one batch and of four): the lowest is reported, a store
+    writes zeros for their pages, a restore leaves the pages of the others alone."""
+    k = kvx()
+    L, N, B, H, D, e, layout, n_used, C, c0, short, ppb = _batches_case(shape, batches, True)
+    spec = oracle.PoolSpec(L, N, B, H, D, e, layout, ppb)
+    T = n_used * B * ppb - short
+    src_np = host_layers(spec, seed=batches)
+    src, host = device_pool(spec, src_np), pinned_chunks(orc, spec, 0, T, C)
+    ctx = ctxs(MODES[mode], 0, getattr(k, flag) if flag else 0, max_ctas)
+    for worst in ([n_used - 1], [2, 3, n_used // 2, n_used - 1], [0, 1, n_used - 2]):
+        table = synth.permuted_table(N // ppb, n_used, seed=17)
+        table[worst] = [N // ppb, -1, np.iinfo(np.int32).max, np.iinfo(np.int32).min][:len(worst)]
+        table_d, dst = torch.from_numpy(table).cuda(), device_pool(spec)
+        torch.cuda.synchronize()
+        k.kv_store(ctx, src, table_d, 0, T, C, host)
+        torch.cuda.synchronize()
+        want, bad = oracle_store(orc, spec, src_np, table, 0, T, C)
+        assert bad == worst[0] and k.kv_get_device_error(ctx) == bad
+        for h, w in zip(host, want):
+            assert first_mismatch(np_of(h), w) is None
+        k.kv_load(ctx, dst, table_d, 0, T, C, host)
+        torch.cuda.synchronize()
+        assert k.kv_get_device_error(ctx) == bad
+        poisoned = [np.full(spec.layer_bytes, POISON, np.uint8) for _ in range(L)]
+        want_l, _ = oracle_load(orc, spec, poisoned, table, 0, T, C, want)
+        for l in range(L):
+            assert first_mismatch(np_of(dst.layers[l]), want_l[l]) is None, l
+
+
 @pytest.mark.parametrize("mode", list(MODES))
 def test_empty_range_is_a_no_op(orc, ctxs, mode):
     k = kvx()
