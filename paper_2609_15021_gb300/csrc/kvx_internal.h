@@ -125,8 +125,8 @@ void set_error_text(const char* text);
 // Launchers (pack_kernels.cu).  Return the cudaError_t of the launch.
 cudaError_t launch_move(int dir, bool link, const MoveParams& p, int grid, cudaStream_t s);
 cudaError_t launch_segments(const SegmentParams& p, int grid, cudaStream_t s);
-// Loads the pack kernels into the current context if lazy loading has not yet.
-cudaError_t load_pack_kernels();
+// Loads the load/store kernels into the current context if lazy loading has not yet.
+cudaError_t load_move_kernels();
 // Bounded waits of the TMA kernels: the limit of each mbarrier wait in SM
 // cycles, the device int set when one expires, and the unit (global index, -1
 // for none) whose load a kernel arms without issuing it (fault point "tma_wait").

@@ -1078,6 +1078,7 @@ kvx_status kv_ctx_create(int device, const kvx_opts* opts, kvx_ctx** out) {
     ctx->queues.resize(kUnitQueues);
     for (uint32_t i = 0; i < kUnitQueues; ++i)
       ctx->queues[i] = {ctx->d_queues + 2 * i, ctx->queue_done_dev + i, 0, 0, 0};
+    if ((e = load_move_kernels()) != cudaSuccess) return fail(e);
     for (int d = 0; d < 2; ++d) ctx->move_occ[d] = link_ctas_per_sm(d);
     ctx->seg_occ = segment_ctas_per_sm();
     if ((e = prepare_tma_kernels()) != cudaSuccess) return fail(e);

@@ -115,7 +115,7 @@ kvx_status scratch_address(int device, uint8_t** out) {
   void* p = nullptr;
   cudaError_t e = cudaGetSymbolAddress(&p, g_scratch);
   if (e != cudaSuccess) return fail_cuda(e, "cudaGetSymbolAddress of the static staging array failed");
-  e = load_pack_kernels();
+  e = load_move_kernels();
   if (e != cudaSuccess) return fail_cuda(e, "loading the pack kernels");
   g_resolved[g_next_entry] = {id, (uint8_t*)p};
   g_next_entry = (g_next_entry + 1) % kCachedContexts;

@@ -213,11 +213,15 @@ cudaError_t launch_move(int dir, bool link, const MoveParams& p, int grid, cudaS
   return cudaGetLastError();
 }
 
-cudaError_t load_pack_kernels() {
+cudaError_t load_move_kernels() {
   // cudaFuncGetAttributes makes CUDA load a kernel that lazy loading has not loaded yet
   cudaFuncAttributes a;
-  const cudaError_t e = cudaFuncGetAttributes(&a, kernel_of(kPack, true));
-  return e == cudaSuccess ? cudaFuncGetAttributes(&a, kernel_of(kPack, false)) : e;
+  for (int dir : {kPack, kUnpack})
+    for (bool link : {false, true}) {
+      const cudaError_t e = cudaFuncGetAttributes(&a, kernel_of(dir, link));
+      if (e != cudaSuccess) return e;
+    }
+  return cudaSuccess;
 }
 
 int link_ctas_per_sm(int dir) {

@@ -6,6 +6,11 @@ zero-copy mode allocates nothing per call.  A captured store/restore is
 replayed twice with new KV written between the replays and each replay is
 checked against the oracle.
 """
+import os
+import subprocess
+import sys
+import time
+
 import numpy as np
 import pytest
 import torch
@@ -158,3 +163,47 @@ def test_first_calls_of_a_context_inside_a_capture(orc):
         assert k.kv_get_device_error(ctx) == -1
     finally:
         k.kv_ctx_destroy(ctx)
+
+
+def _first_device_moves_body():
+    k = kvx()
+    orc = oracle.c_oracle()
+    spec = oracle.PoolSpec(2, 40, 16, 3, 40, 2, oracle.HND)  # page halves of 3,840 B: loads and stores
+    C, T = 64, 37 * 16 - 5
+    src_np, table = host_layers(spec, 51), synth.permuted_table(40, 37, 52)
+    src, dst, tab = device_pool(spec, src_np), device_pool(spec), torch.from_numpy(table).cuda()
+    want, _ = oracle_store(orc, spec, src_np, table, 0, T, C)
+    dev = [torch.full((w.size,), POISON, dtype=torch.uint8, device="cuda") for w in want]
+    ctx = k.kv_ctx_create(0)
+    s, g = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    spin = torch.cuda.Stream()
+    with torch.cuda.graph(g, stream=s):  # global capture mode
+        with torch.cuda.stream(spin):
+            torch.cuda._sleep(2_000_000_000)  # a second of other work on the GPU, outside the capture
+        t = time.perf_counter()
+        k.kv_pack(ctx, src, tab, 0, T, C, dev, stream=s)
+        k.kv_unpack(ctx, dst, tab, 0, T, C, dev, stream=s)
+        t = time.perf_counter() - t
+    assert t < 0.3, f"the first calls took {t:.2f} s: they waited for the GPU"
+    torch.cuda.synchronize()
+    g.replay()
+    torch.cuda.synchronize()
+    loaded, _ = oracle_load(orc, spec, [np.full(spec.layer_bytes, POISON, np.uint8)] * 2, table, 0, T, C, want)
+    for d, w in zip(dev, want):
+        assert first_mismatch(np_of(d), w) is None
+    for t, w in zip(dst.layers, loaded):
+        assert first_mismatch(np_of(t), w) is None
+    assert k.kv_get_device_error(ctx) == -1
+    k.kv_ctx_destroy(ctx)
+    print("FIRST_MOVES_OK")
+
+
+def test_first_device_moves_of_a_process_inside_a_capture():
+    """The context's set-up loads every load/store kernel: a process's first kv_pack and kv_unpack,
+    here in a capture beside other work, load nothing and wait for nothing."""
+    here = os.path.dirname(os.path.abspath(__file__))
+    code = (f"import sys; sys.path[:0] = [{here!r}, {os.path.dirname(here)!r}]; "
+            "import test_graph_gpu as t; t._first_device_moves_body()")
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300, cwd=here)
+    assert r.returncode == 0 and "FIRST_MOVES_OK" in r.stdout, r.stdout[-3000:] + r.stderr[-3000:]
