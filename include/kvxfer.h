@@ -108,12 +108,14 @@ typedef enum {
                                       paper's missing dependency (Sec. 3.2).
                                       Results are then undefined.             */
 /* Device-side moves (kv_pack, kv_unpack, staged mode) use, by default, the
-   TMA kernel when a K or V page half is 8 to 48 KiB: one bulk copy per side where
-   the page half holds its rows in the chunk's order (NHD pools, one head; there
-   from 4 KiB on, in launches below 160 MiB), one tensor-map box per page half for
-   other HND pools, in launches of at least 4 MiB; both staged through shared memory, and measured as fast as the load/store
-   kernel or faster on GB300.  Other page halves, smaller HND launches and HND
-   pools that no tensor map describes use the 16-byte load/store kernel.
+   TMA kernel when a K or V page half is 8 to 48 KiB: one bulk copy per side
+   where the page half holds its rows in the chunk's order (NHD pools, one head;
+   there from 4 KiB on, in launches below 192 MiB), one tensor-map box per page
+   half for other HND pools, in launches of at least 4 MiB; both staged through
+   shared memory.  On GB300 it is as fast as the load/store kernel or faster, but
+   for HND launches of 4 to 24 MiB with page halves above 16 KiB, which take up to
+   4 us more (8 MB: 7.7 us against 4.6).  Other page halves, smaller HND launches
+   and HND pools that no tensor map describes use the 16-byte load/store kernel.
    Zero-copy moves always use the load/store kernel.  The flags below force one of
    them for device-side moves.                                                */
 #define KVX_FLAG_DEVICE_TMA 0x4u   /* TMA everywhere it fits, with one bulk

@@ -428,14 +428,20 @@ kvx_status launch_move_timed(kvx_ctx* ctx, const kvx_pool* P, int dir, int layou
   //   half pages of 4 KiB, 1 GB: 357 / 355 against 324 / 329; of 2 KiB 627 / 619
   //     against 350 / 354: a CTA for each is too little work for its launch, so
   //     half pages below 8 KiB take loads/stores, but flat ones of 4 KiB only
-  //     from 160 MiB on (32 MB 12.9 / 12.9 against 15 / 15, 128 MB 45.7 / 43.6
-  //     against 45.7 / 45.7, 256 MB 88.7 / 88.7 against 82.6 / 84.6)
-  //   HND in replayed graphs, 0.25 / 1 / 2 MB: 3.2 / 4.7 / 6.8 against 2.6 / 3.2 /
-  //     3.3, as a CTA's one box comes in row by row, so launches below 4 MiB take
-  //     loads/stores (8 MB 6.7 against 4.3, 16 MB equal; from 4 MiB on pools of
-  //     such half pages have always had the TMA engine's bounded waits and keep
-  //     them); NHD 2.8 / 3.0 / 3.3, no slower than loads/stores
-  constexpr int64_t kTmaHalf = 8 << 10, kTmaBoxes = 4 << 20, kFlatHalf = 4 << 10, kFlatMost = 160 << 20;
+  //     from 192 MiB on (32 layers of 256-byte rows, 128 MB 42.9 / 41.7 against
+  //     43.1 / 42.8, 184 MB 58.6 / 58.1 against 59.0 / 58.6, 201 MB 64.0 / 63.6
+  //     against 63.6 / 63.6, 216 MB 69.5 / 68.9 against 67.7 / 67.7, 256 MB 85.7 /
+  //     85.4 against 80.0 / 80.1; 62 layers, or half pages of 5 KiB, equal within
+  //     1 % from there to 320 MB and behind at 512 MB: 168.4 / 165.8 against 154.0
+  //     / 155.1)
+  //   HND, 32 KiB half pages, in replayed graphs, 2 / 4 / 8 / 16 / 24 / 32 MB: 4.8 /
+  //     7.3 / 7.7 / 8.7 / 8.3 / 10.2 against 3.4 / 3.6 / 4.6 / 6.9 / 7.9 / 9.7, as a
+  //     CTA's one box comes in row by row; 8 KiB half pages 4.3 / 4.0 / 4.4 / 5.4 /
+  //     7.1 / 8.7 against 3.7 / 3.8 / 4.6 / 6.9 / 8.1 / 10.2.  Launches below 4 MiB
+  //     take loads/stores.  For 32 KiB half pages they are ahead up to 24 MB, but
+  //     from 4 MiB on such pools have always had the TMA engine's bounded waits
+  //     (wait_cycles, KVX_ETIMEOUT) by default, and keep them.
+  constexpr int64_t kTmaHalf = 8 << 10, kTmaBoxes = 4 << 20, kFlatHalf = 4 << 10, kFlatMost = 192 << 20;
   const int64_t unit_bytes = (int64_t)p.B * p.H * p.R;
   const uint32_t f = ctx->opts.flags;
   const bool flat = layout == KVX_LAYOUT_NHD || p.H == 1 || p.B == 1;

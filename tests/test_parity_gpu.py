@@ -650,13 +650,16 @@ def test_noalloc_launches_of_64_chunks(orc, n_chunks, short):
 
 # Where device-side moves change engine: page halves of 4 KiB and 8 KiB less a row, of 4, 8 and 48 KiB
 # and a row more; HND launches just below, at and above 4 MiB; one head and one token per page (whose
-# halves are copied as they lie), with a ragged end.
+# halves are copied as they lie), with a ragged end; halves of 4 KiB just below and above 192 MiB.
 @pytest.mark.parametrize("L,N,B,H,D,e,layout,n_used,C,short", [
-    (2, 40, 15, 2, 128, 2, HND, 37, 60, 7), (2, 40, 16, 2, 128, 2, HND, 37, 64, 7), (2, 40, 16, 2, 128, 2, NHD, 37, 64, 7),
-    (1, 20, 64, 3, 128, 2, HND, 18, 128, 9), (1, 20, 64, 3, 128, 2, NHD, 18, 128, 9), (1, 20, 65, 3, 128, 2, HND, 18, 130, 9),
-    (2, 40, 16, 8, 128, 2, HND, 32, 256, 1), (2, 40, 16, 8, 128, 2, HND, 32, 256, 0), (2, 40, 16, 8, 128, 2, HND, 33, 256, 15),
-    (3, 40, 32, 1, 256, 2, HND, 37, 64, 5), (3, 40, 1, 40, 128, 2, HND, 37, 4, 0),
-    (2, 40, 16, 1, 128, 2, HND, 37, 64, 7), (2, 40, 15, 1, 128, 2, HND, 37, 60, 7), (2, 40, 8, 2, 128, 2, NHD, 37, 64, 7)])
+    (2, 40, 15, 2, 128, 2, HND, 37, 60, 7), (2, 40, 16, 2, 128, 2, HND, 37, 64, 7),
+    (2, 40, 16, 2, 128, 2, NHD, 37, 64, 7), (1, 20, 64, 3, 128, 2, HND, 18, 128, 9),
+    (1, 20, 64, 3, 128, 2, NHD, 18, 128, 9), (1, 20, 65, 3, 128, 2, HND, 18, 130, 9),
+    (2, 40, 16, 8, 128, 2, HND, 32, 256, 1), (2, 40, 16, 8, 128, 2, HND, 32, 256, 0),
+    (2, 40, 16, 8, 128, 2, HND, 33, 256, 15), (3, 40, 32, 1, 256, 2, HND, 37, 64, 5),
+    (3, 40, 1, 40, 128, 2, HND, 37, 4, 0), (2, 40, 16, 1, 128, 2, HND, 37, 64, 7),
+    (2, 40, 15, 1, 128, 2, HND, 37, 60, 7), (2, 40, 8, 2, 128, 2, NHD, 37, 64, 7),
+    (64, 386, 16, 1, 128, 2, HND, 384, 256, 1), (64, 387, 16, 1, 128, 2, NHD, 385, 256, 15)])
 def test_device_engine_borders(orc, ctxs, L, N, B, H, D, e, layout, n_used, C, short):
     k = kvx()
     spec = oracle.PoolSpec(L, N, B, H, D, e, layout)
