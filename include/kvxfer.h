@@ -327,8 +327,12 @@ kvx_status kv_state_load(kvx_ctx* ctx, int32_t num_layers, void* const* layer_ba
  * not let cudaMalloc/cudaFree synchronise the device mid-pipeline.  kv_store
  * needs a context, and a context allocates a staging ring, streams and events.
  * This call creates nothing: it writes mapped host chunks directly over the
- * host link, as kv_store's zero-copy mode does, all on `stream`.  If one of the
- * chunks is not mapped for the GPU, it packs into a static device array of
+ * host link, as kv_store's zero-copy mode does, all on `stream`: one 8-warp CTA
+ * on every other SM until the transfer ends (a caller whose compute should keep
+ * all SMs uses kv_store in KVX_MODE_STAGED, which leaves the transfer to the
+ * copy engines).  If one of the
+ * chunks is not mapped for the GPU (page-locked memory is, where the GPU shares
+ * the host's addresses), it packs into a static device array of
  * KVX_NOALLOC_SCRATCH_BYTES (64 MiB, plus 256 bytes) and copies each packed batch
  * to the host chunks with cudaMemcpyAsync, in stream order (no overlap of packing
  * and copying, unlike kv_store).  Every GPU loading this part of the library
@@ -336,8 +340,8 @@ kvx_status kv_state_load(kvx_ctx* ctx, int32_t num_layers, void* const* layer_ba
  *
  * Arguments, layout, alignment, pinned-memory and range rules are those of
  * kv_store; it runs on the calling thread's current device.  One layer of one
- * chunk (2 * tokens * H * head_dim * elem_bytes) must fit in the array, else
- * KVX_ERANGE (kv_last_error_message names both sizes).
+ * chunk (2 * tokens * H * head_dim * elem_bytes) must fit in the array, mapped
+ * or not, else KVX_ERANGE (kv_last_error_message names both sizes).
  *   dev_first_bad_block : NULL, or a device int64 that the kernel lowers by
  *                         atomicMin to the lowest logical block whose table
  *                         entry is out of range (initialise it, e.g. to
@@ -625,8 +629,10 @@ const char* kv_last_error_message(void);
  * fails with cudaErrorUnknown (cudaErrorMemoryAllocation for "host_alloc")
  * instead of being made.  Points: "launch" (kernel launches), "memcpy"
  * (staged-mode copies), "event" (the staged pipeline's ordering event
- * recorded on the caller's stream), "host_alloc" (kv_host_alloc).  Two more
- * points fail differently.  "tma_wait": the (after_calls + 1)-th next launch
+ * recorded on the caller's stream), "host_alloc" (kv_host_alloc).  Three more
+ * points fail differently.  "chunk_map": the (after_calls + 1)-th next
+ * kv_store_noalloc whose chunks are mapped takes them as not mapped, and
+ * packs and copies.  "tma_wait": the (after_calls + 1)-th next launch
  * of the TMA engine arms the shared-memory stage of its first unit for bytes
  * that no copy brings, so that unit's bounded wait runs out (after
  * kvx_opts.wait_cycles) with no copy in flight: the launch leaves that unit

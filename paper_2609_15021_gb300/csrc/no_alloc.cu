@@ -174,7 +174,7 @@ extern "C" kvx_status kv_store_noalloc(const kvx_pool* pool, const int32_t* bloc
     // zero-copy mode does.  2,048 tokens of a 62-layer pool with 8 heads of 256-byte
     // rows (520 MB) take 2,695 us; packed and copied batch by batch they took 2,923,
     // since a batch's packing waits for the copies of the one before (link: 2,688).
-    if (mapped) {
+    if (mapped && !fault_point("chunk_map")) {
       int sms = 0;
       e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
       if (e != cudaSuccess) return fail_cuda(e, "cudaDeviceGetAttribute");

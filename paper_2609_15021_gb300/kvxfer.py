@@ -439,7 +439,8 @@ def kv_unpack(ctx, pool: KvPool, block_table, tok_begin: int, tok_end: int, chun
 
 def kv_store_noalloc(pool: KvPool, block_table, tok_begin: int, tok_end: int, chunk_tokens: int,
                      host_chunks, dev_first_bad_block=None, stream=None, table_len: int | None = None) -> None:
-    """kv_store for callers that cannot allocate: no context, static device staging (see kvxfer.h)."""
+    """kv_store for callers that cannot allocate: no context; mapped chunks are written directly, others
+    through a static device array (see kvxfer.h)."""
     _check_transfer_tensors(pool, block_table, tok_begin, tok_end, chunk_tokens, host_chunks)
     arr = _ptr_array(host_chunks)
     n_tab = block_table.numel() if table_len is None else table_len

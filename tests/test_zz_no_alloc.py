@@ -3,9 +3,11 @@
 Such callers (an engine whose pool owns all free GPU memory, or code that must
 not let cudaMalloc / cudaFree synchronise the device mid-pipeline) cannot
 create a kvx_ctx, because a context allocates a staging ring, streams and
-events.  kv_store_noalloc packs into a static device array instead.  These
-tests call it through the C ABI and check its chunks byte for byte against
-kv_store's on the same inputs, on two calls in a row (the array keeps the
+events.  kv_store_noalloc writes mapped chunks directly, and packs chunks the
+GPU cannot reach into a static device array that it copies out.  These tests
+call it through the C ABI, on either way (fault point "chunk_map" takes mapped
+chunks as not mapped), and check its chunks byte for byte against kv_store's on
+the same inputs, on two calls in a row (the array, where it is used, keeps the
 previous call's bytes), plus the size limit and the bad-entry report.  Two
 tests run in a fresh process of their own: after the set-up call (an empty
 range), calls leave the GPU's free memory and torch's reserved memory exactly
@@ -32,9 +34,23 @@ pytestmark = pytest.mark.gpu
 
 # (L, N, B, H, D, e, layout, pages used, C, first chunk, t1 short by)
 CALLS = [
-    (62, 48, 16, 8, 128, 2, oracle.HND, 40, 256, 0, 3),   # 62 MiB chunks: two batches, one chunk split
+    (62, 48, 16, 8, 128, 2, oracle.HND, 40, 256, 0, 3),   # 62 MiB chunks: packed, three batches that split chunks
     (2, 64, 16, 2, 64, 2, oracle.NHD, 32, 256, 1, 0),     # small chunks, non-zero start
 ]
+
+
+@pytest.fixture(params=[False, True], ids=["direct", "packed"])
+def store(request):
+    """kv_store_noalloc, its chunks taken as mapped (as they are) or as not mapped."""
+    k = kvx()
+
+    def call(*args, **kw):
+        if request.param:
+            k.kv_fault_inject("chunk_map", 0)
+        k.kv_store_noalloc(*args, **kw)
+
+    yield call
+    k.kv_fault_inject(None)
 
 
 def _expected_via_kv_store(orc, pool, table_d, t0, t1, C, spec):
@@ -49,9 +65,8 @@ def _expected_via_kv_store(orc, pool, table_d, t0, t1, C, spec):
     return [np_of(h) for h in host]
 
 
-def test_noalloc_store_matches_kv_store_twice(orc):
-    k = kvx()
-    for rnd in range(2):  # the same two calls again: the array now holds older bytes
+def test_noalloc_store_matches_kv_store_twice(orc, store):
+    for rnd in range(2):  # the same two calls again: the array, where used, now holds older bytes
         for n_call, case in enumerate(CALLS):
             L, N, B, H, D, e, layout, n_used, C, c0, short = case
             spec = oracle.PoolSpec(L, N, B, H, D, e, layout)
@@ -64,7 +79,7 @@ def test_noalloc_store_matches_kv_store_twice(orc):
             extra = 32
             host = pinned_chunks(orc, spec, t0, t1, C, extra=extra)
             stream = torch.cuda.Stream()
-            k.kv_store_noalloc(pool, table_d, t0, t1, C, host, stream=stream)
+            store(pool, table_d, t0, t1, C, host, stream=stream)
             stream.synchronize()
             for i, (h, w) in enumerate(zip(host, want)):
                 got = np_of(h)
@@ -75,8 +90,7 @@ def test_noalloc_store_matches_kv_store_twice(orc):
                 assert first_mismatch(np_of(h)[:-extra], r) is None
 
 
-def test_noalloc_reports_bad_entries(orc):
-    k = kvx()
+def test_noalloc_reports_bad_entries(orc, store):
     spec = oracle.PoolSpec(2, 16, 16, 2, 64, 2, oracle.HND)
     src_np = host_layers(spec, seed=8)
     pool = device_pool(spec, src_np)
@@ -85,7 +99,7 @@ def test_noalloc_reports_bad_entries(orc):
     table_d = torch.from_numpy(table).cuda()
     err = torch.full((1,), np.iinfo(np.int64).max, dtype=torch.int64, device="cuda")
     host = pinned_chunks(orc, spec, 0, 192, 64)
-    k.kv_store_noalloc(pool, table_d, 0, 192, 64, host, dev_first_bad_block=err)
+    store(pool, table_d, 0, 192, 64, host, dev_first_bad_block=err)
     torch.cuda.synchronize()
     assert int(err.item()) == 7
     want, bad = oracle_store(orc, spec, src_np, table, 0, 192, 64)
@@ -121,7 +135,7 @@ def _run_fresh(body: str, marker: str):
 def _allocation_free_body():
     k = kvx()
     orc = oracle.c_oracle()
-    # 62 MiB chunks: every call packs two batches and splits one chunk
+    # 62 MiB chunks: a packed call makes three batches and splits chunks
     spec = oracle.PoolSpec(62, 48, 16, 8, 128, 2, oracle.HND)
     src_np = host_layers(spec, seed=700)
     pool = device_pool(spec, src_np)
@@ -135,7 +149,11 @@ def _allocation_free_body():
     k.kv_store_noalloc(pool, table_d, 0, 0, 256, host, stream=stream)  # set-up only: empty range
     torch.cuda.synchronize()
     free0, reserved0 = torch.cuda.mem_get_info()[0], torch.cuda.memory_reserved()
-    for _ in range(2):
+    for packed in (False, True, False, True):
+        if packed:
+            k.kv_fault_inject("chunk_map", 0)
+        for h in host:
+            h.fill_(POISON)
         k.kv_store_noalloc(pool, table_d, 0, t1, 256, host, stream=stream)
         stream.synchronize()
         free, reserved = torch.cuda.mem_get_info()[0], torch.cuda.memory_reserved()
