@@ -627,7 +627,9 @@ const char* kv_last_error_message(void);
  * Host-side fault injection for testing error handling without faulting a
  * GPU: the (after_calls + 1)-th next CUDA call at `point` in this process
  * fails with cudaErrorUnknown (cudaErrorMemoryAllocation for "host_alloc")
- * instead of being made.  Points: "launch" (kernel launches), "memcpy"
+ * instead of being made.  Points: "launch" (kernel launches), "queue_launch"
+ * (those whose warps take their work from a queue: large kv_store / kv_load
+ * launches over the host link), "memcpy"
  * (staged-mode copies), "event" (the staged pipeline's ordering event
  * recorded on the caller's stream), "host_alloc" (kv_host_alloc).  Three more
  * points fail differently.  "chunk_map": the (after_calls + 1)-th next

@@ -489,6 +489,8 @@ kvx_status launch_move_timed(kvx_ctx* ctx, const kvx_pool* P, int dir, int layou
   else if (tma)
     KVX_CUDA_AT("launch", launch_move_tma(dir, flat ? KVX_LAYOUT_NHD : KVX_LAYOUT_HND, p, (int)grid, stage_bytes,
                                           stages, wt, s));
+  else if (queue)
+    KVX_CUDA_AT("launch", fault_now("queue_launch") ? cudaErrorUnknown : launch_move(dir, over_link, p, (int)grid, s));
   else
     KVX_CUDA_AT("launch", launch_move(dir, over_link, p, (int)grid, s));
   if (queue) {
@@ -1189,8 +1191,8 @@ kvx_status kv_state_load(kvx_ctx* ctx, int32_t num_layers, void* const* layer_ba
 }
 
 kvx_status kv_fault_inject(const char* point, int32_t after_calls) {
-  static const char* const points[] = {"launch",    "memcpy",   "event",    "host_alloc",
-                                       "tier_exit", "tma_wait", "chunk_map"};
+  static const char* const points[] = {"launch",    "queue_launch", "memcpy",   "event",
+                                       "host_alloc", "tier_exit",    "tma_wait", "chunk_map"};
   std::lock_guard<std::mutex> lock(g_fault_mu);
   if (!point || !point[0]) {
     g_fault_point[0] = 0;

@@ -169,44 +169,107 @@ def test_where_the_unit_queue_begins(orc, ctxs, shape, batches, full):
     _run_case(orc, ctxs(2, 0, 0, 1), _batches_case(shape, batches, full), torch.cuda.Stream())
 
 
-def test_unit_queues_serve_launch_after_launch(orc):
-    """Launches over the host link of at least eight units a warp take their units from
-    counters that the launch before left at zero (a context keeps 1,280 of them).  With one
-    CTA a 512 KiB transfer does: more launches than counters, on two streams at once, a
-    captured one (which takes no counters) replayed among them, and every byte as it should be."""
-    k = kvx()
-    spec = oracle.PoolSpec(2, 40, 16, 4, 128, 2, HND)
-    T, C = 37 * 16 - 5, 256
-    src_np, table = host_layers(spec, 71), synth.permuted_table(40, 37, 72)
-    want, _ = oracle_store(orc, spec, src_np, table, 0, T, C)
-    poisoned = [np.full(spec.layer_bytes, POISON, np.uint8) for _ in range(2)]
-    want_l, _ = oracle_load(orc, spec, poisoned, table, 0, T, C, want)
-    src, table_d = device_pool(spec, src_np), torch.from_numpy(table).cuda()
-    hosts = [pinned_chunks(orc, spec, 0, T, C) for _ in range(2)]
-    dsts = [device_pool(spec) for _ in range(2)]
-    streams = [torch.cuda.Stream() for _ in range(2)]
-    ctx = k.kv_ctx_create(0, max_ctas=1)
-    try:
+UNIT_QUEUES = 1280  # counter pairs of a context, used in turn
+
+
+class _QueueRig:
+    """Two pools with different bytes behind one table, and what storing and restoring each gives.
+    One CTA and 1.3 MB: every launch takes its units from a queue, if a counter pair is free."""
+
+    def __init__(self, orc):
+        self.k = k = kvx()
+        spec = oracle.PoolSpec(2, 24, 16, 4, 128, 2, HND)
+        self.T, self.C = 20 * 16 - 5, 256
+        table = synth.permuted_table(24, 20, 72)
+        src_np = [host_layers(spec, seed) for seed in (71, 73)]
+        self.want = [oracle_store(orc, spec, a, table, 0, self.T, self.C)[0] for a in src_np]
+        poisoned = [np.full(spec.layer_bytes, POISON, np.uint8) for _ in range(2)]
+        loaded = [oracle_load(orc, spec, poisoned, table, 0, self.T, self.C, w)[0] for w in self.want]
+        self.loaded = [[torch.from_numpy(a).cuda() for a in layers] for layers in loaded]
+        self.src, self.table = [device_pool(spec, a) for a in src_np], torch.from_numpy(table).cuda()
+        self.hosts = [pinned_chunks(orc, spec, 0, self.T, self.C) for _ in range(4)]
+        self.dsts = [device_pool(spec) for _ in range(2)]
+        self.ctx = k.kv_ctx_create(0, max_ctas=1)
         torch.cuda.synchronize()
+
+    def store(self, which, host, **kw):
+        self.k.kv_store(self.ctx, self.src[which], self.table, 0, self.T, self.C, host, **kw)
+
+    def load(self, dst, host, **kw):
+        self.k.kv_load(self.ctx, dst, self.table, 0, self.T, self.C, host, **kw)
+
+    def stored(self, which, host):
+        return all(np.array_equal(np_of(h), w) for h, w in zip(host, self.want[which]))
+
+    def restored(self, which, dst):
+        return all(torch.equal(t, w) for t, w in zip(dst.layers, self.loaded[which]))
+
+
+def test_unit_queues_serve_launch_after_launch(orc):
+    """Each counter pair of a context serves launch after launch: the counters only count up, from
+    values the host knows, and a launch gets a pair once the one before it is done.  Over three
+    times through the pairs, every launch but those of the first time is compared, and moves other
+    bytes than the buffer held.  The fault point counts the launches that got a queue: all of
+    them did, the next one fails, which leaves its pair usable."""
+    q = _QueueRig(orc)
+    k = q.k
+    try:
+        for which in (0, 1):
+            for h, w in zip(q.hosts[2 + which], q.want[which]):
+                h.numpy()[:] = w
+        k.kv_fault_inject("queue_launch", 3 * UNIT_QUEUES)
+        for i in range(3 * UNIT_QUEUES // 2):
+            which = i % 2
+            q.store(which, q.hosts[0])
+            q.load(q.dsts[0], q.hosts[2 + which])
+            if i == UNIT_QUEUES // 2:
+                torch.cuda.synchronize()  # from here on each launch finds the one before on its pair done
+            if i >= UNIT_QUEUES // 2:
+                torch.cuda.synchronize()
+                assert q.stored(which, q.hosts[0]) and q.restored(which, q.dsts[0]), i
+            elif i % 64 == 0:
+                torch.cuda.synchronize()
+        with pytest.raises(k.KvxError) as e:
+            q.store(0, q.hosts[0])
+        assert e.value.status == k.KVX_ECUDA
+        torch.cuda.synchronize()
+        assert q.stored(1, q.hosts[0])
+        k.kv_fault_inject("queue_launch", UNIT_QUEUES)
+        for i in range(UNIT_QUEUES):  # once more through the pairs, the one of the failed launch among them
+            q.store(i % 2, q.hosts[0])
+            torch.cuda.synchronize()
+            assert q.stored(i % 2, q.hosts[0]), i
+        with pytest.raises(k.KvxError):
+            q.store(0, q.hosts[0])
+        assert k.kv_get_device_error(q.ctx) == -1
+    finally:
+        k.kv_fault_inject(None)
+        k.kv_ctx_destroy(q.ctx)
+
+
+def test_unit_queues_on_two_streams_and_a_graph(orc):
+    """More launches than counter pairs, on two streams at once, a captured one (which takes no
+    pair) replayed among them; the buffers change with every launch, and hold the last one's bytes."""
+    q = _QueueRig(orc)
+    k = q.k
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    try:
         graph = torch.cuda.CUDAGraph()
         with torch.cuda.graph(graph, stream=streams[0]):
-            k.kv_store(ctx, src, table_d, 0, T, C, hosts[0])
+            q.store(0, q.hosts[0])
         for i in range(350):
-            for s, host, dst in zip(streams, hosts, dsts):
-                k.kv_store(ctx, src, table_d, 0, T, C, host, stream=s)
-                k.kv_load(ctx, dst, table_d, 0, T, C, host, stream=s)
+            for s, host, dst in zip(streams, q.hosts, q.dsts):
+                q.store(i % 2, host, stream=s)
+                q.load(dst, host, stream=s)
             if i % 50 == 0:
                 with torch.cuda.stream(streams[0]):
                     graph.replay()
         torch.cuda.synchronize()
-        for host, dst in zip(hosts, dsts):
-            for h, w in zip(host, want):
-                assert first_mismatch(np_of(h), w) is None
-            for l in range(2):
-                assert first_mismatch(np_of(dst.layers[l]), want_l[l]) is None
-        assert k.kv_get_device_error(ctx) == -1
+        for host, dst in zip(q.hosts, q.dsts):
+            assert q.stored(1, host) and q.restored(1, dst)
+        assert k.kv_get_device_error(q.ctx) == -1
     finally:
-        k.kv_ctx_destroy(ctx)
+        k.kv_ctx_destroy(q.ctx)
 
 
 @pytest.mark.parametrize("name", ["ragged_tail_offset_start", "27b_shape_two_chunks", "fp8_1568_token_chunks"])
