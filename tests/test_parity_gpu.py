@@ -146,7 +146,8 @@ def test_load_store_units(orc, ctxs, name, mode, flag, max_ctas):
 
 
 # Launches over the link whose units come from a queue, with one CTA (eight warps): bytes of the
-# whole range, in 4 KiB batches, where the queue begins (a restore at 32 batches, a store at 64).
+# whole range, in 4 KiB batches, where the queue begins (a restore at 32 batches, a store at 64), and
+# where its units become two, three, four and eight batches.  Device-side, where they become two.
 # Rows, pages and planes that batches cut anywhere: rows of 192 B in HND, of 80 B in NHD, one-head
 # pages of 288 B in logical blocks of seven.
 UNIT_SHAPES = {"hnd_192B_rows": (2, 16, 3, 96, 2, HND, 1), "nhd_80B_rows": (2, 8, 5, 40, 2, NHD, 1),
@@ -163,10 +164,17 @@ def _batches_case(shape, batches, full):
 
 
 @pytest.mark.parametrize("full", [False, True])
-@pytest.mark.parametrize("batches", [32, 64])
+@pytest.mark.parametrize("batches", [32, 64, 384, 576, 768, 4096])
 @pytest.mark.parametrize("shape", list(UNIT_SHAPES))
-def test_where_the_unit_queue_begins(orc, ctxs, shape, batches, full):
+def test_units_from_the_queue(orc, ctxs, shape, batches, full):
     _run_case(orc, ctxs(2, 0, 0, 1), _batches_case(shape, batches, full), torch.cuda.Stream())
+
+
+@pytest.mark.parametrize("full", [False, True])
+@pytest.mark.parametrize("shape", list(UNIT_SHAPES))
+def test_device_units_of_two_batches(orc, ctxs, shape, full):
+    L, N, B, H, D, e, layout, n_used, C, c0, short, ppb = case = _batches_case(shape, 8193, full)
+    _run_case(orc, ctxs(1, 2 * C * H * D * e * L, kvx().KVX_FLAG_DEVICE_LSU), case, torch.cuda.Stream())
 
 
 UNIT_QUEUES = 1280  # counter pairs of a context, used in turn
