@@ -846,7 +846,7 @@ def run_shared(args, world, rank, local):
         link_bytes = kern[dom]["bytes_per_launch"] / 2
         achieved = link_bytes / (kern[dom]["avg_launch_ms"] * 1e-3) / GB
         peak, which = link_ceiling(link, sm_link, direction)
-        roofline = {"bound": "host_link", "kernel": f"move_kernel<{dom},HND> (zero-copy), rank 0",
+        roofline = {"bound": "host_link", "kernel": f"move_kernel<{dom},link> (zero-copy, HND), rank 0",
                     "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                     "traffic": recorded_traffic(s).get(f"zerocopy_{dom}", link_bytes),
                     "peak_source": f"rank 0's GPU before the timed steps, {direction}: copy engines (pinned "
@@ -1119,8 +1119,8 @@ def run_ours(args):
             link_bytes = kern[dom]["bytes_per_launch"] / 2
             achieved = link_bytes / (kern[dom]["avg_launch_ms"] * 1e-3) / GB
             peak, which = link_ceiling(link, sm_link, direction)
-            roofline = {"bound": "host_link", "kernel": f"move_kernel<{dom},{LAY}> (zero-copy)", "achieved": achieved,
-                        "peak": peak, "unit": "GB/s", "frac": achieved / peak,
+            roofline = {"bound": "host_link", "kernel": f"move_kernel<{dom},link> (zero-copy, {LAY})",
+                        "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                         "traffic": traffic.get(f"zerocopy_{dom}", link_bytes),
                         "peak_source": f"the larger of two host-link ceilings measured in this run, {direction}: "
                                        f"copy engines (pinned cudaMemcpyAsync of 1 GiB) {link[direction]:.1f} GB/s, "
@@ -1178,7 +1178,7 @@ def run_ours(args):
             nl, per_launch, ms = legs[tma][d]
             achieved = per_launch / (ms * 1e-3) / GB
             kname = ((f"tmap_move_kernel<{name}>" if args.layout == "hnd" else f"tma_move_kernel<{name},NHD>")
-                     if tma else f"move_kernel<{name},{LAY}>")
+                     if tma else f"move_kernel<{name},device>")
             hbm_roofline[name] = {"kernel": f"{kname} (device chunks)", "achieved": achieved,
                                   "frac": achieved / hbm_peak, "launches": nl,
                                   "algorithmic_bytes_per_launch": per_launch, "avg_launch_ms": ms,

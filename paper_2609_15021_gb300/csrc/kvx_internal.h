@@ -122,7 +122,8 @@ int64_t cut_units(MoveParams* p, bool link, int64_t queue_warps);
 int64_t chunk_bytes(const kvx_pool* P, const Geometry& g, int64_t tokens);
 void set_error_text(const char* text);
 
-// Launchers (pack_kernels.cu).  Return the cudaError_t of the launch.
+// Launchers (pack_kernels.cu).  Return the cudaError_t of the launch.  link: the
+// chunks are mapped host memory.
 cudaError_t launch_move(int dir, bool link, const MoveParams& p, int grid, cudaStream_t s);
 cudaError_t launch_segments(const SegmentParams& p, int grid, cudaStream_t s);
 // Loads the load/store kernels into the current context if lazy loading has not yet.

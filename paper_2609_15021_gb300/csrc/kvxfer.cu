@@ -423,10 +423,11 @@ kvx_status launch_move_timed(kvx_ctx* ctx, const kvx_pool* P, int dir, int layou
   // pools, one head, one token); loads/stores otherwise (per-row bulk copies of
   // HND pages without tensor maps are slower).  Measured on GB300 (us, TMA
   // against loads/stores, pack and unpack of 16-token bf16 pages):
-  //   half pages of 8 KiB or more, 1 GB: HND 32 KiB 301 / 297 against 302 / 298,
-  //     8 KiB 312 / 306 against 312 / 314; NHD 32 KiB 300 / 296 against 300 / 296
-  //   half pages of 4 KiB, 1 GB: 357 / 355 against 324 / 329; of 2 KiB 627 / 619
-  //     against 350 / 354: a CTA for each is too little work for its launch, so
+  //   half pages of 8 KiB or more, 1 GB: HND 32 KiB 298 / 295 against 297 / 296,
+  //     8 KiB 309 / 305 against 309 / 311; NHD 32 KiB 297 / 295 against 297 / 294,
+  //     8 KiB 306 / 303 against 308 / 311; 32 MB, any of them, 10 against 11 to 12
+  //   half pages of 4 KiB, 1 GB: 346 / 345 against 321 / 326; of 2 KiB 602 / 602
+  //     against 349 / 357: a CTA for each is too little work for its launch, so
   //     half pages below 8 KiB take loads/stores, but flat ones of 4 KiB only
   //     from 192 MiB on (32 layers of 256-byte rows, 128 MB 42.9 / 41.7 against
   //     43.1 / 42.8, 184 MB 58.6 / 58.1 against 59.0 / 58.6, 201 MB 64.0 / 63.6
@@ -575,7 +576,6 @@ struct Plan {
   const kvx_pool* P;
   Geometry g;
   const int32_t* table;
-  int32_t C;
   int64_t first_chunk;  // chunk index of the first chunk of the range
   int64_t n;            // chunks in the range
   int64_t bpc;          // pages per chunk (C / B)
@@ -816,7 +816,6 @@ kvx_status transfer(kvx_ctx* ctx, const kvx_pool* P, const int32_t* table, int64
   if (st != KVX_OK || n == 0) return st;
   pl.P = P;
   pl.table = table;
-  pl.C = C;
   pl.first_chunk = t0 / C;
   pl.n = n;
   pl.bpc = C / P->block_tokens;

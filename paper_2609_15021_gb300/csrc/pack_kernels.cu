@@ -39,8 +39,8 @@ constexpr int64_t kBatchesApart = 8192;
 // Taken from a queue, a unit is up to 4 batches as long as every warp gets 24
 // units, and 8 where every warp gets 64 of these (the last units end apart).  A
 // 32k-token restore of the 27B shape (8.3 GB) takes 39,377 us with 8, 39,391 with
-// 4, 39,430 with 1 and 39,419 with 32; 400 MB 2,095 us with 4, 2,097 with 8 and
-// 2,110 with 32; storing one chunk (65 MB) 342 us with 1, 344 with 4, 346 with 8.
+// 4, 39,430 with 1 and 39,419 with 32; storing 400 MB 2,095 us with 4, 2,097 with 8
+// and 2,110 with 32, one chunk (65 MB) 342 us with 1, 344 with 4, 346 with 8.
 constexpr int64_t kQueueBatches = 4, kQueueUnits = 24;
 constexpr int64_t kLargeBatches = 8, kLargeUnits = 64;
 
@@ -59,18 +59,22 @@ __device__ __forceinline__ uint64_t div_by(uint64_t n, const FastDiv& f) {
 // or up to 4955 (a store 5295 or up to 5370), depending on the GPU and the
 // number of CTAs; taking units from a queue it takes 4846 to 4849 (5294) on all
 // of them, with 48 CTAs as with 96.
-// Measured on GB300, one launch, 32 layers, 16-token HND pages, 8 heads of
-// head_dim 128 bf16 unless stated; in brackets the same call when a unit was a
+// Measured on GB300, launches back to back, 32 layers, 16-token HND pages, 8 heads
+// of head_dim 128 bf16 unless stated; in brackets the same call when a unit was a
 // page half, read row by row (vector by vector where a row was no power of two):
-//   restore over the link, 1 GB: 4848 us, 0.999 of the copy engines' 211.6 GB/s
-//     (4853 to 4890); head_dim 96, 256 MB: 1221 us (1335); one 128-byte head:
-//     1227 us (1263)
-//   restore, 4 MB: 27 us (32; head_dim 96: 107); 1 MB: 13 us (19; 60), since 4 KiB
-//     units put 256 warps on 1 MB where 32 of them made eight round trips each
-//   store over the link, 1 GB: 5294 us, 0.999 of 193.5 GB/s (5296); head_dim 96,
-//     256 MB: 1329 us (1508); one 128-byte head: 1334 us (1455)
-//   pack / unpack in device memory, 1 GB: 300 / 298 us, 6.8 TB/s (308 / 310);
-//     head_dim 96: 304 / 304 us (476 / 451); one 128-byte head: 350 / 354 (606 / 600)
+//   restore over the link, 1 GB: 4736 us (4741); head_dim 96, 256 MB: 1217 us
+//     (1331); one 128-byte head: 1223 us (1260)
+//   restore, 4 MB: 24 us (28; head_dim 96: 24, 104); 1 MB: 8 us (17; 10, 57), since
+//     4 KiB units put 256 warps on 1 MB where 32 of them made eight round trips each
+//   store over the link, 1 GB: 5168 us (5169); head_dim 96, 256 MB: 1326 us (1492);
+//     one 128-byte head: 1332 us (1414); 1 MB 9 us (8; head_dim 96: 10, 27)
+//   pack / unpack in device memory, 1 GB: 297 / 296 us, 6.9 TB/s (305 / 307);
+//     head_dim 96: 300 / 303 us (478 / 452); one 128-byte head: 350 / 357 (609 / 608)
+//   the same of NHD pages, whose halves were straight copies (32 KiB unless stated;
+//     the TMA engine takes them unless told not to), 16 MB: 8 / 8 us (9 / 9), 64 MB,
+//     which L2 holds: 21 / 21 (19 / 19), 1 GB: 297 / 293 (305 / 305); halves of 8 KiB,
+//     16 MB: 8 / 8 (6 / 6), 1 GB: 307 / 310 (307 / 304); of 128 KiB (this kernel's by
+//     default), 16 MB: 8 / 8 (14 / 14), 64 MB: 21 / 21 (32 / 33), 1 GB: 295 / 293 (309 / 309)
 // Dealt out in advance over the link a unit is one batch: units of eight took 4945
 // us for the 1 GB restore and 5370 for the store, and equal shares of 26,368 B, so
 // that a warp's last batch is not whole, 95 us for a 16 MB restore instead of 83.

@@ -1,14 +1,14 @@
 // tma_kernels.cu -- device-side pack / unpack with the Tensor Memory
 // Accelerator (TMA), staged through shared memory.
 //
-// Same work units and byte mapping as move_kernel (pack_kernels.cu): one
-// (chunk, layer, page, K|V) unit at a time, here per CTA of one warp.  A unit
-// is copied global -> shared with completion on an mbarrier, then shared ->
-// global tracked as a bulk group; registers never hold the data.  By default
-// every unit gets its own CTA with a single stage (six 32 KiB CTAs fit an SM,
-// and the block scheduler keeps DRAM busy as CTAs finish); a grid capped by
-// the caller strides each CTA over many units through a ring of stages, so
-// the loads of the next units overlap the store of the current one.
+// Same byte mapping as move_kernel (pack_kernels.cu), but a unit is one page
+// half, (chunk, layer, page, K|V), moved by a CTA of one warp.  A unit is copied
+// global -> shared with completion on an mbarrier, then shared -> global tracked
+// as a bulk group; registers never hold the data.  By default every unit gets
+// its own CTA with a single stage (six 32 KiB CTAs fit an SM, and the block
+// scheduler keeps DRAM busy as CTAs finish); a grid capped by the caller strides
+// each CTA over many units through a ring of stages, so the loads of the next
+// units overlap the store of the current one.
 //
 // Two ways to move the page side of an HND unit (its [head][token][row]
 // bytes, which the chunk holds in [token][head][row] order):
@@ -113,8 +113,9 @@ struct Unit {
   int page;
 };
 
-// Same decode as move_kernel; a bad table entry zero-fills the chunk rows
-// (pack) with ordinary stores and reports the logical block.  lane < 0: a
+// Unit u of the launch: plane by plane, (layer, K|V) of a chunk, its page halves in
+// token order.  A bad table entry zero-fills the chunk rows (pack) with ordinary
+// stores and reports the logical block.  lane < 0: a
 // second decode of the same unit (store side), which repeats no side effect.
 template <int DIR>
 __device__ __forceinline__ Unit decode(const MoveParams& p, int64_t u, int& j, int64_t& job_begin, int lane) {
@@ -348,7 +349,8 @@ bool encode_tensor_maps(const kvx_pool* P, int64_t row_bytes, void* out) {
 // driver attribute calls.
 cudaError_t prepare_tma_kernels() {
   cudaError_t e = cudaSuccess;
-  for (cudaError_t r : {set_smem(tma_move_kernel<kPack, KVX_LAYOUT_HND>), set_smem(tma_move_kernel<kPack, KVX_LAYOUT_NHD>),
+  for (cudaError_t r : {set_smem(tma_move_kernel<kPack, KVX_LAYOUT_HND>),
+                        set_smem(tma_move_kernel<kPack, KVX_LAYOUT_NHD>),
                         set_smem(tma_move_kernel<kUnpack, KVX_LAYOUT_HND>),
                         set_smem(tma_move_kernel<kUnpack, KVX_LAYOUT_NHD>), set_smem(tmap_move_kernel<kPack>),
                         set_smem(tmap_move_kernel<kUnpack>)})

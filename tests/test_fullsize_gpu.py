@@ -115,7 +115,8 @@ def _check_sampled(orc, spec, ctx_tokens, src_layers, dst_layers, ta, tb, chunks
 def test_fullsize_device_pack_unpack_sampled(orc, engine):
     """The benchmark's HBM leg at 128k tokens: kv_pack into device chunks and
     kv_unpack into a poisoned pool, in the launch configuration bench.py times
-    (64 chunks per launch, one CTA or warp per 32 KiB unit)."""
+    (64 chunks per launch; one CTA per 32 KiB page half, or a warp for two 4 KiB
+    batches)."""
     k = kvx()
     ctx_tokens, pool_blocks = 131072, 10240
     spec = oracle.PoolSpec(L, pool_blocks, B, H, D, E, oracle.HND)
